@@ -97,6 +97,7 @@ struct mm_ctx {
     bool own_stream = false;
     int nsm = 0;
     int blocks = 0;
+    int threads = 0;
     int blocks_per_sm_req = 0;
     const void* kernel = nullptr;
     std::string err;
@@ -823,16 +824,17 @@ int build_hierarchy(mm_ctx* ctx, mm::Problem& P, HostCsr A) {
     return MM_OK;
 }
 
-// The solver kernel built for `variant` blocks per SM and its grid (as many
-// blocks as are co-resident, at most variant per SM).
+// The solver kernel built for `variant` x 256 threads per SM and its grid:
+// one block of that size per SM.
 int select_kernel(mm_ctx* ctx, int variant) {
     ctx->kernel = mm::solver_kernel(variant);
+    ctx->threads = mm::solver_threads(variant);
     int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, ctx->kernel, MM_BLOCK, 0) != cudaSuccess || bps < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, ctx->kernel, ctx->threads, 0) != cudaSuccess || bps < 1) {
         cudaGetLastError();
         return MM_ERR_CUDA;
     }
-    ctx->blocks = std::min(bps, variant) * ctx->nsm;
+    ctx->blocks = ctx->nsm;
     return MM_OK;
 }
 
@@ -852,7 +854,7 @@ int launch_solver(mm_ctx* ctx, int mode, const mm::Params& prm) {
     CK_CUDA(cudaMemsetAsync(ctx->P.err, 0, sizeof(int), ctx->stream));
     void* args[] = {(void*)&ctx->P};
     CK_CUDA(cudaEventRecord(ctx->ev0, ctx->stream));
-    CK_CUDA(cudaLaunchCooperativeKernel(ctx->kernel, dim3(ctx->blocks), dim3(MM_BLOCK), args, 0, ctx->stream));
+    CK_CUDA(cudaLaunchCooperativeKernel(ctx->kernel, dim3(ctx->blocks), dim3(ctx->threads), args, 0, ctx->stream));
     CK_CUDA(cudaEventRecord(ctx->ev1, ctx->stream));
     CK_CUDA(cudaMemcpyAsync(ctx->h_state, ctx->d_state, sizeof(mm::DevState), cudaMemcpyDeviceToHost,
                             ctx->stream));
@@ -969,6 +971,8 @@ const void* solver_kernel(int min_blocks) {
     }
 }
 
+int solver_threads(int min_blocks) { return 256 * (min_blocks == 2 || min_blocks == 4 ? min_blocks : 3); }
+
 const void* solver_batch_kernel(int min_blocks) {
     return min_blocks == 4 ? solver_batch_kernel_4() : min_blocks == 2 ? solver_batch_kernel_2() : solver_batch_kernel_3();
 }
@@ -989,6 +993,7 @@ int ctx_view(mm_ctx* ctx, CtxView* out) {
     out->ident = ctx->d_ident;
     out->has_mesh = ctx->has_mesh;
     out->kernel = ctx->kernel;
+    out->threads = ctx->threads;
     out->d_state = ctx->d_state;
     out->nnz_mag = ctx->nnzm_true;
     out->nnz_phi = ctx->nnzp_true;

@@ -14,7 +14,9 @@
 #pragma once
 #include <cstdint>
 
-#define MM_BLOCK 256
+#ifndef MM_BLOCK
+#define MM_BLOCK 256          // threads per block (solver units set their own)
+#endif
 #define MM_SELL 32
 #define MM_MAXRED 16          // reduction values per phase
 #define MM_NSLOT 3            // state slots: current, trial t, trial s
@@ -216,6 +218,7 @@ struct CtxView {
     const unsigned char* ident;  // device
     bool has_mesh;
     const void* kernel;          // the solver kernel the context launches
+    int threads;                 // and its threads per block
     DevState* d_state;           // device
     long long nnz_mag, nnz_phi;  // true nonzeros of the two graphs
 };
@@ -225,8 +228,10 @@ struct CtxView {
 struct mm_ctx;
 namespace mm {
 // Device function pointer of the solver kernel built for at least
-// min_blocks resident blocks per SM (2, 3 or 4; others -> 3).
+// min_blocks x 256 resident threads per SM (2, 3 or 4; others -> 3), and the
+// threads per block it is launched with (min_blocks x 256: one block per SM).
 const void* solver_kernel(int min_blocks);
+int solver_threads(int min_blocks);
 // The batched solver kernel (teams of blocks, one problem per team);
 // min_blocks 3 or 4 (others -> 3).
 const void* solver_batch_kernel(int min_blocks);

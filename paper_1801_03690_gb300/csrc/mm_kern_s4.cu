@@ -1,4 +1,6 @@
-// Single-problem solver kernel for at least 4 resident blocks per SM.
+// Single-problem solver kernel for at least 4 x 256 resident threads per SM,
+// as one block.
+#define MM_BLOCK 1024
 #include "mm_solver_body.cuh"
 
 namespace mm {

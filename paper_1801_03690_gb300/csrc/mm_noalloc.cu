@@ -193,7 +193,7 @@ extern "C" int mm_energy_gradient_noalloc(mm_ctx* ctx, const double* m_dev, cons
                                                    v.field_T[1] * hs, v.field_T[2] * hs, bad);
     if ((e = cudaGetLastError()) != cudaSuccess) return mm::ctx_fail(ctx, MM_ERR_CUDA, cudaGetErrorString(e));
     void* args[] = {(void*)&Q};
-    if ((e = cudaLaunchCooperativeKernel(v.kernel, dim3(v.blocks), dim3(MM_BLOCK), args, 0, st)) != cudaSuccess)
+    if ((e = cudaLaunchCooperativeKernel(v.kernel, dim3(v.blocks), dim3(v.threads), args, 0, st)) != cudaSuccess)
         return mm::ctx_fail(ctx, MM_ERR_CUDA, cudaGetErrorString(e));
     if (grad_dev &&
         (e = cudaMemsetAsync(grad_dev, 0, (size_t)v.n_nodes * 3 * sizeof(double), st)) != cudaSuccess)

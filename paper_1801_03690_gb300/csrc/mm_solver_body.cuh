@@ -4,8 +4,8 @@
 //
 // One cooperative launch covers a whole minimisation.  The blocks form a
 // team that moves through phases separated by team barriers; every phase is
-// a grid-stride pass over rows (one thread per SELL-32 row) that also writes
-// per-block partial sums.  After a barrier every block reduces the same
+// a pass over rows (one thread per SELL-32 row) that also writes per-block
+// partial sums.  After a barrier every block reduces the same
 // partials in the same fixed order, so all blocks hold bit-identical scalars
 // and take the same branch at every decision (potential-solve convergence,
 // li1-li3, line-search branches, beta*ZA, t1-t3) without host round trips or
@@ -23,13 +23,37 @@ namespace {
 
 constexpr unsigned long long kBarrierTimeoutNs = 5000000000ull;  // 5 s per wait
 constexpr int kWarps = MM_BLOCK / 32;
+constexpr int kFlat = 4;         // team_reduce: values summed through shared memory at most
+
+// A block's share of `items` (32-row slices, or rows that take a whole warp):
+// full rounds, in which the team's warps take items in turn, and its part of
+// the last, partial round, `count` items from `tail` on.  Turns spread the
+// expensive rows (magnet surface, grain boundaries) over all blocks:
+// contiguous ranges left a block waiting 7 to 9 us at the barriers of a step on
+// 3.2 M unknowns.  Splitting the last round evenly keeps every SM at work on a
+// mesh with fewer rows than threads (29,791 rows: 6 or 7 warps on each of
+// the 152 SMs instead of 16 on 58 of them).
+struct Share {
+    int full, tail, count;
+};
+
+struct TeamSmem {
+    double v[kFlat][MM_BLOCK];       // one value per thread
+    double w[MM_MAXRED][kWarps];     // one value per warp
+    double res[MM_MAXRED];           // the team's values
+    Share phi, nm, phi4;             // slices of the potential rows, magnetic rows, float4 groups of the former
+    Share rows[MM_MAXLEV], coarse[MM_MAXLEV], dense;   // multigrid: slices of a level, its restriction's items, dense rows
+    int dead;
+};
 
 struct Team {
     int nb;
     int rank;
     unsigned long long* count;   // arrival counter (barrier words [0..1])
+    unsigned long long target;   // its value once the last barrier is complete
     int* err;
     double* part;
+    TeamSmem* sm;
     int epoch;
     bool dead;
 };
@@ -40,169 +64,222 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Team barrier with a bounded wait.  The arrival counter is 64-bit and only
-// grows (zeroed by the host before each launch): a block's k-th barrier is
-// complete once the counter reaches k * nb, so the last arriver publishes
-// completion with its own increment and no reset or second word is needed
-// (measured on GB300: 1.9 us per empty barrier with a reset counter and a
-// generation word).  The fences make each block's writes before the barrier
+// Arrival and wait of one thread per block.  The 64-bit counter only grows
+// (zeroed by the host before each launch): the k-th barrier is complete once
+// it reaches k * nb.  A release-add publishes the block's writes (those of
+// its other threads are ordered before it by the block barrier) and an
+// acquire-load that sees the target makes every other block's visible.  The
+// wait is bounded: it ends with the device error flag set, which the other
+// blocks' waits look at now and then.  What bounds it is the chain of L2
+// round trips (write drain, add, load), so there is nothing else in it:
+// an atomic with its result, two full fences, a sleep and a look at the
+// error flag on each side took 1.91 us per empty barrier at 304 blocks of
+// 256 threads and 2.35 us at 608; this form takes 1.25 us at 152 x 512 and
+// 1.29 us at 152 x 1024 (one block per SM) and 1.42 / 2.28 us at the old
+// grids.  An all-gather of tagged values without a counter took 3.2 us and
+// more (every block polls every other's line).
+__device__ __forceinline__ bool team_arrive_wait(Team& t) {
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(t.count), "l"(1ull) : "memory");
+    unsigned long long seen;
+    unsigned spin = 0;
+    unsigned long long t0 = 0;
+    while (true) {
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(t.count) : "memory");
+        if (seen >= t.target) return true;
+        if ((++spin & 1023u) == 0) {
+            if (*(volatile int*)t.err) return false;
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kBarrierTimeoutNs) {
+                atomicCAS(t.err, 0, (int)ST_TIMEOUT);
+                return false;
+            }
+        }
+    }
+}
+
+// Team barrier with a bounded wait: the writes of every block before it are
 // visible to every block after it.
 __device__ bool team_sync(Team& t) {
-    __shared__ int s_err;
+    t.target += (unsigned long long)t.nb;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile int* verr = t.err;
-        int e = *verr;
-        if (e == 0) {
-            const unsigned long long nb = (unsigned long long)t.nb;
-            __threadfence();
-            const unsigned long long old = atomicAdd(t.count, 1ull);
-            const unsigned long long target = (old / nb + 1ull) * nb;
-            if (old + 1ull != target) {
-                volatile unsigned long long* vc = t.count;
-                const unsigned long long t0 = global_ns();
-                while (*vc < target) {
-                    if (*verr) break;
-                    __nanosleep(32);
-                    if (global_ns() - t0 > kBarrierTimeoutNs) {
-                        atomicCAS(t.err, 0, (int)ST_TIMEOUT);
-                        break;
-                    }
-                }
-            }
-            __threadfence();
-            e = *verr;
-        }
-        s_err = e;
-    }
+    if (threadIdx.x == 0 && !team_arrive_wait(t)) t.sm->dead = 1;
     __syncthreads();
-    t.dead = (s_err != 0);
+    t.dead = t.sm->dead != 0;
     return !t.dead;
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
+__device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     return v;
 }
 
-__device__ __forceinline__ double warp_max(double v) {
+// Sum (or maximum) of N values in a fixed order, as a tree: the FP64 adder
+// answers after 64 cycles and takes a warp every 19, so depth counts.
+template <int N>
+__device__ __forceinline__ double fold_tree(double (&a)[N], bool sum) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
+    for (int h = 1; h < N; h *= 2) {
+#pragma unroll
+        for (int i = 0; i + h < N; i += 2 * h) a[i] = sum ? a[i] + a[i + h] : fmax(a[i], a[i + h]);
+    }
+    return a[0];
+}
+
+// Over the lanes of a warp; the result is lane 0's.
+template <int LANES = 32>
+__device__ __forceinline__ double warp_fold(double v, bool sum) {
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        const double u = __shfl_down_sync(0xffffffffu, v, o);
+        v = sum ? v + u : fmax(v, u);
+    }
     return v;
 }
 
-// Reduce NS sums and NX maxima over the team.  Deterministic: fixed order
-// within warps (shfl_down tree, lane 0), across warps (ascending) and across
-// blocks (ascending strided accumulation, then the same block tree).
-template <typename AT>
-__device__ __forceinline__ AT warp_sum_t(AT v) {
+// Sums of KP (a power of two, at most 32) values over the lanes of a warp in
+// KP - 1 + log2(32 / KP) additions: a pair of lanes shares each round's work,
+// one keeping the lower half of the values and the other the upper half.
+// The sum of value k ends in lane (32 / KP) * k.
+template <int KP>
+__device__ __forceinline__ double warp_sums_shared(double (&v)[KP]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
+    for (int n = KP / 2; n >= 1; n /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double give = up ? v[i] : v[i + n];
+            const double keep = up ? v[i + n] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+        o >>= 1;
+    }
+#pragma unroll
+    for (int r = 16 / KP; r > 0; r >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], r);
+    return v[0];
 }
 
-template <typename AT>
-__device__ __forceinline__ AT warp_max_t(AT v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// AT is the type of the per-thread and per-warp accumulation (float for the
-// FP32 phases, whose sums are all of positive terms); the combination across
-// warps and blocks is always FP64.
-template <int NS, int NX, typename AT = double>
-__device__ bool team_reduce(Team& t, AT (&s)[NS > 0 ? NS : 1], AT (&x)[NX > 0 ? NX : 1]) {
-    static_assert(NS + NX <= MM_MAXRED, "too many reduction values");
-    __shared__ double sh[MM_MAXRED][kWarps];
-    __shared__ double res[MM_MAXRED];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        AT v = warp_sum_t<AT>(s[k]);
-        if (lane == 0) sh[k][warp] = (double)v;
-    }
-#pragma unroll
-    for (int k = 0; k < NX; ++k) {
-        AT v = warp_max_t<AT>(x[k]);
-        if (lane == 0) sh[NS + k][warp] = (double)v;
-    }
-    __syncthreads();
-    double* part = t.part + (size_t)(t.epoch & 1) * MM_MAXRED * t.nb;
-    if (threadIdx.x < NS + NX) {
-        const int k = threadIdx.x;
-        double a = sh[k][0];
-        for (int w = 1; w < kWarps; ++w) a = (k < NS) ? a + sh[k][w] : fmax(a, sh[k][w]);
-        part[(size_t)k * t.nb + t.rank] = a;
-    }
-    t.epoch++;
+// Second half of a team reduction: the block's partial values of K
+// quantities (the first NS sums, the others maxima) are in `part`; after the
+// barrier every block folds all partials identically, one warp per quantity,
+// into t.sm->res.
+template <int K, int NS>
+__device__ __forceinline__ bool team_combine(Team& t, const double* part) {
     if (!team_sync(t)) return false;
-    // every block folds all partials identically
-#pragma unroll
-    for (int k = 0; k < NS + NX; ++k) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = warp; k < K; k += kWarps) {
         const double* pk = part + (size_t)k * t.nb;
-        double a = (k < NS) ? 0.0 : 0.0;
-        for (int j = threadIdx.x; j < t.nb; j += MM_BLOCK) a = (k < NS) ? a + pk[j] : fmax(a, pk[j]);
-        a = (k < NS) ? warp_sum(a) : warp_max(a);
-        if (lane == 0) sh[k][warp] = a;
-    }
-    __syncthreads();
-    if (threadIdx.x < NS + NX) {
-        const int k = threadIdx.x;
-        double a = sh[k][0];
-        for (int w = 1; w < kWarps; ++w) a = (k < NS) ? a + sh[k][w] : fmax(a, sh[k][w]);
-        res[k] = a;
-    }
-    __syncthreads();
+        const bool sum = k < NS;
+        double s = 0.0;                       // the maxima are of values >= 0
+        for (int j0 = 0; j0 < t.nb; j0 += 5 * 32) {
+            double a[5];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) s[k] = (AT)res[k];
-#pragma unroll
-    for (int k = 0; k < NX; ++k) x[k] = (AT)res[NS + k];
+            for (int u = 0; u < 5; ++u) {
+                const int j = j0 + 32 * u + lane;
+                a[u] = j < t.nb ? pk[j] : 0.0;
+            }
+            const double f = fold_tree<5>(a, sum);
+            s = j0 == 0 ? f : sum ? s + f : fmax(s, f);
+        }
+        s = warp_fold(s, sum);
+        if (lane == 0) t.sm->res[k] = s;
+    }
     __syncthreads();
     return true;
 }
 
-// Team sums accumulated in FP32 per thread and warp, returned in FP64.
+// Partials of this reduction (double buffered: a block may enter the next
+// reduction while others still fold this one).
+__device__ __forceinline__ double* team_partials(Team& t) {
+    double* p = t.part + (size_t)(t.epoch & 1) * MM_MAXRED * t.nb;
+    t.epoch++;
+    return p;
+}
+
+// Reduce NS sums and NX maxima (of values >= 0) over the team, in FP64 and in
+// a fixed order.  FP64 additions are what it costs: a full shuffle tree in
+// every warp for every value issues 5 additions a warp, 80 per block and
+// value pair, and took 7.6 us for two values (5.3 us for one) with the serial
+// folds that followed.  Up to kFlat values therefore go through shared
+// memory, where one warp per value sums MM_BLOCK / 32 of them per lane before
+// its only tree; more values share their trees (warp_sums_shared).
+template <int NS, int NX>
+__device__ bool team_reduce(Team& t, double (&s)[NS > 0 ? NS : 1], double (&x)[NX > 0 ? NX : 1]) {
+    constexpr int K = NS + NX;
+    static_assert(K <= MM_MAXRED, "too many reduction values");
+    TeamSmem& sm = *t.sm;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* part = team_partials(t);
+    if constexpr (K <= kFlat) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) sm.v[k][threadIdx.x] = s[k];
+#pragma unroll
+        for (int k = 0; k < NX; ++k) sm.v[NS + k][threadIdx.x] = x[k];
+        __syncthreads();
+        if (warp < K) {
+            const bool sum = warp < NS;
+            double f = 0.0;
+#pragma unroll 1
+            for (int h = 0; h < kWarps; h += 8) {
+                double a[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) a[u] = sm.v[warp][32 * (h + u) + lane];
+                const double g = fold_tree<8>(a, sum);
+                f = h == 0 ? g : sum ? f + g : fmax(f, g);
+            }
+            f = warp_fold(f, sum);
+            if (lane == 0) part[(size_t)warp * t.nb + t.rank] = f;
+        }
+    } else {
+        constexpr int KP = NS > 8 ? 16 : NS > 4 ? 8 : NS > 2 ? 4 : NS > 1 ? 2 : 1;
+        double v[KP];
+#pragma unroll
+        for (int k = 0; k < KP; ++k) v[k] = k < NS ? s[k < NS ? k : 0] : 0.0;
+        const double f = warp_sums_shared<KP>(v);
+        constexpr int step = 32 / KP;
+        if (lane % step == 0 && lane / step < NS) sm.w[lane / step][warp] = f;
+#pragma unroll
+        for (int k = 0; k < NX; ++k) {
+            const double m = warp_fold(x[k], false);
+            if (lane == 0) sm.w[NS + k][warp] = m;
+        }
+        __syncthreads();
+        for (int k = warp; k < K; k += kWarps) {
+            const double f2 = warp_fold(lane < kWarps ? sm.w[k][lane] : 0.0, k < NS);
+            if (lane == 0) part[(size_t)k * t.nb + t.rank] = f2;
+        }
+    }
+    if (!team_combine<K, NS>(t, part)) return false;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) s[k] = sm.res[k];
+#pragma unroll
+    for (int k = 0; k < NX; ++k) x[k] = sm.res[NS + k];
+    return true;
+}
+
+// Team sums accumulated in FP32 per thread and warp (the FP32 phases, whose
+// sums are all of positive terms), in FP64 across warps and blocks.
 template <int NS>
 __device__ bool team_sum_f32(Team& t, float (&s)[NS], double (&out)[NS]) {
-    __shared__ double sh[MM_MAXRED][kWarps];
-    __shared__ double res[MM_MAXRED];
+    TeamSmem& sm = *t.sm;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* part = team_partials(t);
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
-        const float v = warp_sum_t<float>(s[k]);
-        if (lane == 0) sh[k][warp] = (double)v;
+        const float v = warp_sum(s[k]);
+        if (lane == 0) sm.w[k][warp] = (double)v;
     }
     __syncthreads();
-    double* part = t.part + (size_t)(t.epoch & 1) * MM_MAXRED * t.nb;
-    if (threadIdx.x < NS) {
-        const int k = threadIdx.x;
-        double a = sh[k][0];
-        for (int w = 1; w < kWarps; ++w) a += sh[k][w];
-        part[(size_t)k * t.nb + t.rank] = a;
+    if (warp < NS) {
+        const double f = warp_fold(lane < kWarps ? sm.w[warp][lane] : 0.0, true);
+        if (lane == 0) part[(size_t)warp * t.nb + t.rank] = f;
     }
-    t.epoch++;
-    if (!team_sync(t)) return false;
+    if (!team_combine<NS, NS>(t, part)) return false;
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        const double* pk = part + (size_t)k * t.nb;
-        double a = 0.0;
-        for (int j = threadIdx.x; j < t.nb; j += MM_BLOCK) a += pk[j];
-        a = warp_sum(a);
-        if (lane == 0) sh[k][warp] = a;
-    }
-    __syncthreads();
-    if (threadIdx.x < NS) {
-        const int k = threadIdx.x;
-        double a = sh[k][0];
-        for (int w = 1; w < kWarps; ++w) a += sh[k][w];
-        res[k] = a;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NS; ++k) out[k] = res[k];
-    __syncthreads();
+    for (int k = 0; k < NS; ++k) out[k] = sm.res[k];
     return true;
 }
 
@@ -217,7 +294,28 @@ __device__ __forceinline__ Row sell_row(const long long* sptr, int r) {
     return {b + (r & 31), (int)((sptr[s + 1] - b) >> 5)};
 }
 
-#define ROWS(r, n) for (int r = t.rank * MM_BLOCK + (int)threadIdx.x; r < (n); r += t.nb * MM_BLOCK)
+__device__ __forceinline__ Share make_share(const Team& t, int items) {
+    const int stride = t.nb * kWarps, full = items / stride, left = items - full * stride;
+    const int q = left / t.nb, m = left - q * t.nb;
+    return {full, full * stride + q * t.rank + min(t.rank, m), q + (t.rank < m ? 1 : 0)};
+}
+
+// Item of this warp in round k = 0 .. full (-1: none).
+__device__ __forceinline__ int team_item(const Team& t, const Share& h, int k) {
+    const int warp = (int)(threadIdx.x >> 5);
+    if (k < h.full) return (k * t.nb + t.rank) * kWarps + warp;
+    return warp < h.count ? h.tail + warp : -1;
+}
+
+// Loop over this warp's items of a share (warp-uniform), and over this
+// thread's rows r < n of a share of slices.
+#define ITEMS(i, share)                                                       \
+    for (int i##_k = 0, i##_f = (share).full; i##_k <= i##_f; ++i##_k)        \
+        if (const int i = team_item(t, (share), i##_k); i >= 0)
+#define ROWS(r, share, n)                                                     \
+    ITEMS(r##_s, share)                                                       \
+        if (const int r = 32 * r##_s + ((int)threadIdx.x & 31); r < (n))
+
 // Row dot products over a SELL-32 row.  All column indices and values of a
 // chunk are loaded before any gather, so each thread keeps a whole row's
 // worth of independent loads in flight: measured on GB300 this lifts an FP32
@@ -225,8 +323,10 @@ __device__ __forceinline__ Row sell_row(const long long* sptr, int r) {
 // entries are read once per product, so they are loaded with the
 // evict-first (streaming) policy, which leaves L2 to the gathered vectors
 // (+1.5% NCG iterations/s on the 8.7 M-unknown polycrystal).
-// Lanes past the row's width read x[pad] (pad = r for square matrices, 0
-// for rectangular ones whose row index may exceed the columns).
+// Entries past the slice's width (the same for the whole warp) gather x[pad]
+// (pad = r for square matrices, 0 for rectangular ones whose row index may
+// exceed the columns) and skip the FP64 multiply-add, which would occupy the
+// SM's FP64 pipe for 19 cycles to add zero.
 template <int CH, typename T, typename VT, typename XT>
 __device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const int* __restrict__ col,
                                       const VT* __restrict__ val, const XT* x, int r, int pad) {
@@ -243,7 +343,10 @@ __device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const 
             v[u] = ok ? __ldcs(val + e) : VT(0);
         }
 #pragma unroll
-        for (int u = 0; u < CH; ++u) s += (T)v[u] * (T)x[c[u]];
+        for (int u = 0; u < CH; ++u) {
+            const T g = (T)x[c[u]];
+            if (sizeof(T) == 4 || k0 + u < A.width) s += (T)v[u] * g;
+        }
     }
     return s;
 }
@@ -275,14 +378,17 @@ __device__ __forceinline__ void sell_dot3(const long long* __restrict__ sptr, co
         }
 #pragma unroll
         for (int u = 0; u < CH; ++u) {
-            s0 += v[u] * x[c[u]];
-            s1 += v[u] * x[n + c[u]];
-            s2 += v[u] * x[2 * n + c[u]];
+            const T g0 = x[c[u]], g1 = x[n + c[u]], g2 = x[2 * n + c[u]];
+            if (sizeof(T) == 4 || k0 + u < A.width) {
+                s0 += v[u] * g0;
+                s1 += v[u] * g1;
+                s2 += v[u] * g2;
+            }
         }
     }
 }
 
-// Two SELL-32 rows r0 and r1 = r0 + team stride (two: r1 exists) per thread,
+// Two SELL-32 rows r0 and r1 of different slices (two: r1 exists) per thread,
 // CH entries of both rows loaded before any gather: twice the loads in
 // flight of the one-row form at the register cost of CH = 16.  Used by the
 // FP32 direction step and the level-0 products of the multigrid cycle,
@@ -366,7 +472,7 @@ __device__ __forceinline__ float sell_dot_tab(const long long* __restrict__ sptr
                                               const float* __restrict__ val, const int* __restrict__ tab,
                                               const float* x, int r) {
     const SliceTab ta = slice_tab(tab, r);
-    if (ta.d[0] == MM_NO_TAB) return sell_dot<16, float>(sptr, col, val, x, r, r);
+    if (ta.d[0] == MM_NO_TAB) return sell_dot<16, float>(sptr, col, val, x, r);
     const Row A = sell_row(sptr, r);
     float v[8];
 #pragma unroll
@@ -377,17 +483,21 @@ __device__ __forceinline__ float sell_dot_tab(const long long* __restrict__ sptr
     return s;
 }
 
-// Grid-stride loop over row pairs (r, r2 = r + team stride); two: r2 < n.
-#define ROWS2(r, r2, two, n)                                                                     \
-    for (int r = t.rank * MM_BLOCK + (int)threadIdx.x, r2 = 0; r < (n); r += 2 * t.nb * MM_BLOCK) \
-        if (const bool two = ((r2 = r + t.nb * MM_BLOCK) < (n)); true)
+// Loop over row pairs (r, r2): the rows of two rounds per thread; two: r2
+// exists.
+#define ROWS2(r, r2, two, share, n)                                                                          \
+    for (int r##_k = 0, r##_f = (share).full, r2 = 0; r##_k <= r##_f; r##_k += 2)                            \
+        if (const int r##_s = team_item(t, (share), r##_k); r##_s >= 0)                                      \
+            if (const int r = 32 * r##_s + ((int)threadIdx.x & 31); r < (n))                                 \
+                if (const int r##_t = r##_k < r##_f ? team_item(t, (share), r##_k + 1) : -1; true)           \
+                    if (const bool two = r##_t >= 0 && (r2 = 32 * r##_t + ((int)threadIdx.x & 31)) < (n); true)
 
 // The FP32 products of level 0 (K_phi and the smoothed prolongation) over the
 // team's rows in the tile shape P.tile_rows selects; f(r, s, v) takes row r,
 // its sum s and v = pre(r), the row's vector operands, which pre loads before
 // the product's loads are issued: the vector loads then overlap the matrix
 // loads and the gathers instead of following them.  Both shapes visit a
-// thread's rows in the same order (r, r + stride, r + 2 stride, ...), so
+// thread's rows in the same order (its rows of the rounds), so
 // per-thread sums f accumulates come out in the same order too.  tab: the
 // slice offset tables of the FP32 K_phi (nullptr for other matrices).
 // pad_self: lanes past a row's width gather x[r] (square matrices) rather
@@ -398,7 +508,7 @@ __device__ __forceinline__ void level0_products(const Problem& P, const Team& t,
                                                 const int* __restrict__ tab, const float* x, int n, bool pad_self,
                                                 Pre pre, F f) {
     if (P.tile_rows != 1) {
-        ROWS2(r, r2, two, n) {
+        ROWS2(r, r2, two, t.sm->phi, n) {
             const auto v0 = pre(r);
             const auto v1 = pre(two ? r2 : r);
             float s0, s1;
@@ -408,7 +518,7 @@ __device__ __forceinline__ void level0_products(const Problem& P, const Team& t,
             if (two) f(r2, s1, v1);
         }
     } else {
-        ROWS(r, n) {
+        ROWS(r, t.sm->phi, n) {
             const auto v0 = pre(r);
             f(r, tab ? sell_dot_tab(sptr, col, val, tab, x, r) : sell_dot<16, float>(sptr, col, val, x, r, pad_self ? r : 0),
               v0);
@@ -439,7 +549,10 @@ __device__ __forceinline__ double row_div(const Problem& P, const double* x, int
             b2[u] = ok ? __ldg(P.B + 2 * nz + e) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) bp += b0[u] * x[c[u]] + b1[u] * x[nm + c[u]] + b2[u] * x[2 * nm + c[u]];
+        for (int u = 0; u < 8; ++u) {
+            const double g0 = x[c[u]], g1 = x[nm + c[u]], g2 = x[2 * nm + c[u]];
+            if (k0 + u < mr.width) bp += b0[u] * g0 + b1[u] * g1 + b2[u] * g2;
+        }
     }
     return bp;
 }
@@ -463,12 +576,13 @@ __device__ __forceinline__ void row_divT(const Problem& P, const double* phi, in
             q2[u] = ok ? __ldg(P.G + 2 * nz + e) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const double ph = phi[c[u]];
-            t0 += q0[u] * ph;
-            t1 += q1[u] * ph;
-            t2 += q2[u] * ph;
-        }
+        for (int u = 0; u < 8; ++u)
+            if (k0 + u < rw.width) {
+                const double ph = phi[c[u]];
+                t0 += q0[u] * ph;
+                t1 += q1[u] * ph;
+                t2 += q2[u] * ph;
+            }
     }
 }
 
@@ -513,7 +627,7 @@ __device__ bool ph_trial(Ctx& C, int c, int s, double a) {
     double dummy[1] = {0.0};
     const double* xc = P.X[c];
     double* xs = P.X[s];
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
         double u0 = xc[i] + a * P.d[i];
         double u1 = xc[nm + i] + a * P.d[nm + i];
         double u2 = xc[2 * nm + i] + a * P.d[2 * nm + i];
@@ -541,7 +655,7 @@ __device__ bool ph_pinit(Ctx& C, int s, double& bb, double& rz, double& rr) {
     const double* x = P.X[s];
     double acc[3] = {0.0, 0.0, 0.0};
     double dummy[1] = {0.0};
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         const double kphi = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, P.phi, p);
         double bp = 0.0;
         if (p < nm) {
@@ -567,7 +681,7 @@ __device__ bool ph_pinit(Ctx& C, int s, double& bb, double& rz, double& rr) {
 __device__ bool ph_pmatvec(Ctx& C, const double* v, double* q) {
     const Problem& P = *C.P;
     Team& t = C.t;
-    ROWS(p, P.nphi) q[p] = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, v, p);
+    ROWS(p, t.sm->phi, P.nphi) q[p] = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, v, p);
     return team_sync(t);
 }
 
@@ -579,7 +693,7 @@ __device__ bool ph_pdirection(Ctx& C, const double* z, double beta, double* d, d
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
     const bool first = (beta == 0.0);
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         const double s = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, z, p);
         const double dn = first ? z[p] : z[p] + beta * d[p];
         const double qn = first ? s : s + beta * q[p];
@@ -598,7 +712,7 @@ __device__ bool ph_pupdate(Ctx& C, const double* v, double a, double& rz, double
     Team& t = C.t;
     double acc[2] = {0.0, 0.0};
     double dummy[1] = {0.0};
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         P.phi[p] += a * v[p];
         const double r = P.pres[p] - a * P.pq[p];
         const double z = r * P.dinvP[p];
@@ -616,7 +730,7 @@ __device__ bool ph_pupdate(Ctx& C, const double* v, double a, double& rz, double
 __device__ bool ph_pzero(Ctx& C) {
     const Problem& P = *C.P;
     Team& t = C.t;
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         P.phi[p] = 0.0;
         P.pres[p] = 0.0;
     }
@@ -715,10 +829,9 @@ __device__ __forceinline__ void amg_restrict_g(const Problem& P, const Team& t, 
     float* xn = last ? nullptr : P.lev[l + 1].x;
     const float* dn = last ? nullptr : P.lev[l + 1].dinv;
     const float on = last ? 0.0f : P.lev[l + 1].omega;
-    const int lane = threadIdx.x & 31, wpb = MM_BLOCK / 32, nw = t.nb * wpb;
-    const int gw = t.rank * wpb + (int)(threadIdx.x >> 5), grp = lane / G, gl = lane % G;
-    for (int I0 = gw * RPW; I0 < V.nc; I0 += nw * RPW) {
-        const int I = I0 + grp;
+    const int lane = threadIdx.x & 31, grp = lane / G, gl = lane % G;
+    ITEMS(I0, t.sm->coarse[l]) {
+        const int I = I0 * RPW + grp;
         const float s = group_csr_dot2<G, 12>(V.t_ptr, V.t_col, V.t_val, bx, I < V.nc ? I : -1, gl);
         if (gl == 0 && I < V.nc) {
             bn[I] = s;
@@ -727,16 +840,23 @@ __device__ __forceinline__ void amg_restrict_g(const Problem& P, const Team& t, 
     }
 }
 
-// Levels with few, long restriction rows (the coarse end of the hierarchy:
-// hundreds of entries per row, a few hundred rows) take a whole warp per
-// row, the others a group of P.restrict_lanes lanes, 8 by default (measured
-// on the 8.7 M-unknown polycrystal: 8 lanes 190 us, 4 lanes 211, 16 lanes
-// 225 for the level-0 down phase).
+// Lanes per restriction row.  Levels with long rows (the coarse end of the
+// hierarchy: hundreds of entries) or with no more rows than the team has
+// warps take a whole warp per row, the others P.restrict_lanes lanes, 8 by
+// default (measured on the 8.7 M-unknown polycrystal: 8 lanes 190 us, 4 lanes
+// 211, 16 lanes 225 for the level-0 down phase).
+__device__ __forceinline__ int restrict_group(const Problem& P, const Team& t, int l) {
+    const Level& V = P.lev[l];
+    if (V.wide || (P.restrict_lanes == 0 && V.nc <= t.nb * kWarps)) return 32;
+    return P.restrict_lanes == 4 || P.restrict_lanes == 16 ? P.restrict_lanes : 8;
+}
+
 template <class XF>
 __device__ __forceinline__ void amg_restrict(const Problem& P, const Team& t, const Level& V, int l, XF bx) {
-    if (V.wide) amg_restrict_g<32>(P, t, V, l, bx);
-    else if (P.restrict_lanes == 4) amg_restrict_g<4>(P, t, V, l, bx);
-    else if (P.restrict_lanes == 16) amg_restrict_g<16>(P, t, V, l, bx);
+    const int g = restrict_group(P, t, l);
+    if (g == 32) amg_restrict_g<32>(P, t, V, l, bx);
+    else if (g == 4) amg_restrict_g<4>(P, t, V, l, bx);
+    else if (g == 16) amg_restrict_g<16>(P, t, V, l, bx);
     else amg_restrict_g<8>(P, t, V, l, bx);
 }
 
@@ -763,7 +883,7 @@ __device__ __noinline__ bool ph_amg_down(Ctx& C, int l) {
     if (l == 0) {
         amg_down0_rows(P, t);
     } else {
-        ROWS(r, V.n) V.rpre[r] = V.b[r] - sell_dot<16, float>(V.sptr, V.col, V.val, V.x, r);
+        ROWS(r, t.sm->rows[l], V.n) V.rpre[r] = V.b[r] - sell_dot<16, float>(V.sptr, V.col, V.val, V.x, r);
     }
     if (!team_sync(t)) return false;
     const float* rp = V.rpre;
@@ -776,13 +896,12 @@ __device__ __noinline__ bool ph_amg_dense(Ctx& C) {
     const Problem& P = *C.P;
     Team& t = C.t;
     const int n = P.nco, lane = threadIdx.x & 31;
-    const int wpb = MM_BLOCK / 32;
-    for (int row = t.rank * wpb + (int)(threadIdx.x >> 5); row < n; row += t.nb * wpb) {
+    ITEMS(row, t.sm->dense) {
         const float* a = P.ainv + (size_t)row * n;
         float s = 0.0f;
 #pragma unroll 8
         for (int j = lane; j < n; j += 32) s += a[j] * P.bco[j];
-        s = warp_sum_t<float>(s);
+        s = warp_sum(s);
         if (lane == 0) P.yco[row] = s;
     }
     return team_sync(t);
@@ -811,7 +930,7 @@ __device__ __noinline__ bool ph_amg_up(Ctx& C, int l, double& rz, double& rr) {
     if (l == 0) {
         level0_products(P, t, V.u_sptr, V.u_col, V.u_val, nullptr, yc, V.n, false, pre, row);
     } else {
-        ROWS(r, V.n) {
+        ROWS(r, t.sm->rows[l], V.n) {
             const float2 v = pre(r);
             row(r, sell_dot<16, float>(V.u_sptr, V.u_col, V.u_val, yc, r, 0), v);
         }
@@ -844,7 +963,7 @@ __device__ bool ph_p32_init(Ctx& C, double& rz, double& rr) {
     const Problem& P = *C.P;
     Team& t = C.t;
     if (use_amg(P)) {
-        ROWS(p, P.nphi) {
+        ROWS(p, t.sm->phi, P.nphi) {
             const float r = (float)P.pres[p];
             P.pres32[p] = r;
             P.amg_x0[p] = P.amg_omega * P.dinvP32[p] * r;
@@ -855,7 +974,7 @@ __device__ bool ph_p32_init(Ctx& C, double& rz, double& rr) {
     }
     float acc[2] = {0.0f, 0.0f};
     double out[2];
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         const float r = (float)P.pres[p];
         const float z = r * P.dinvP32[p];
         P.pres32[p] = r;
@@ -912,14 +1031,14 @@ __device__ bool ph_p32_update(Ctx& C, float a, double& rz, double& rr) {
         // no sums here: r.z and |r|^2 come with z from the V-cycle
         float4* __restrict__ x04 = reinterpret_cast<float4*>(P.amg_x0);
         const float om = P.amg_omega;
-        ROWS(i, n4) {
+        ROWS(i, t.sm->phi4, n4) {
             const float4 d = dir4[i], q = q4[i], r = res4[i], e = del4[i], w = dv4[i];
             const float4 nr = make_float4(r.x - a * q.x, r.y - a * q.y, r.z - a * q.z, r.w - a * q.w);
             del4[i] = make_float4(e.x + a * d.x, e.y + a * d.y, e.z + a * d.z, e.w + a * d.w);
             res4[i] = nr;
             x04[i] = make_float4(om * w.x * nr.x, om * w.y * nr.y, om * w.z * nr.z, om * w.w * nr.w);
         }
-        ROWS(j, P.nphi - 4 * n4) {
+        if (const int j = (int)threadIdx.x; t.rank == t.nb - 1 && j < P.nphi - 4 * n4) {
             const int p = 4 * n4 + j;
             P.pdelta32[p] += a * P.pdir32[p];
             const float r = P.pres32[p] - a * P.pq32[p];
@@ -932,7 +1051,7 @@ __device__ bool ph_p32_update(Ctx& C, float a, double& rz, double& rr) {
     float acc[2] = {0.0f, 0.0f};
     double out[2];
     float4* __restrict__ z4 = reinterpret_cast<float4*>(P.pprec32);
-    ROWS(i, n4) {
+    ROWS(i, t.sm->phi4, n4) {
         const float4 d = dir4[i], q = q4[i], r = res4[i], e = del4[i], w = dv4[i];
         const float4 nr = make_float4(r.x - a * q.x, r.y - a * q.y, r.z - a * q.z, r.w - a * q.w);
         const float4 z = make_float4(nr.x * w.x, nr.y * w.y, nr.z * w.z, nr.w * w.w);
@@ -942,7 +1061,7 @@ __device__ bool ph_p32_update(Ctx& C, float a, double& rz, double& rr) {
         acc[0] += (nr.x * z.x + nr.y * z.y) + (nr.z * z.z + nr.w * z.w);
         acc[1] += (nr.x * nr.x + nr.y * nr.y) + (nr.z * nr.z + nr.w * nr.w);
     }
-    ROWS(j, P.nphi - 4 * n4) {
+    if (const int j = (int)threadIdx.x; t.rank == t.nb - 1 && j < P.nphi - 4 * n4) {
         const int p = 4 * n4 + j;
         P.pdelta32[p] += a * P.pdir32[p];
         const float r = P.pres32[p] - a * P.pq32[p];
@@ -965,7 +1084,7 @@ __device__ bool ph_p64_refine(Ctx& C, double& rr) {
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
     const float* dl = P.pdelta32;
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         const double s = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, dl, p);
         P.phi[p] += (double)dl[p];
         const double r = P.pres[p] - s;
@@ -1065,7 +1184,7 @@ __device__ bool ph_gradient(Ctx& C, int s, bool trial) {
     // sums: exchange, anisotropy, Zeeman, phi.rhs, phi.r, dphi, M0, M1, M2, sum w
     double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     double mx[1] = {0.0};
-    ROWS(p, P.nphi) {
+    ROWS(p, t.sm->phi, P.nphi) {
         acc[4] += P.phi[p] * P.pres[p];
         P.PHI[s][p] = P.phi[p];
         if (p < nm) {
@@ -1124,14 +1243,14 @@ __device__ bool ph_phi_start(Ctx& C, int c, int ref, double theta) {
     Team& t = C.t;
     const double* a = P.PHI[c];
     const double* b = P.PHI[ref];
-    ROWS(p, P.nphi) P.phi[p] = (theta == 0.0) ? a[p] : a[p] + theta * (b[p] - a[p]);
+    ROWS(p, t.sm->phi, P.nphi) P.phi[p] = (theta == 0.0) ? a[p] : a[p] + theta * (b[p] - a[p]);
     return team_sync(t);
 }
 
 __device__ bool ph_phi_restore(Ctx& C, int c) {
     const Problem& P = *C.P;
     Team& t = C.t;
-    ROWS(p, P.nphi) P.phi[p] = P.PHI[c][p];
+    ROWS(p, t.sm->phi, P.nphi) P.phi[p] = P.PHI[c][p];
     return team_sync(t);
 }
 
@@ -1163,7 +1282,7 @@ __device__ bool ph_hess(Ctx& C, int s, const double* v, double ca, double beta, 
     const bool first = (beta == 0.0);
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
         double c0, c1, c2, k0, k1, k2;
         row_local(P, v, i, c0, c1, c2, k0, k1, k2);
         const double v0 = v[i], v1 = v[nm + i], v2 = v[2 * nm + i];
@@ -1219,9 +1338,9 @@ __device__ bool ph_operator(Ctx& C, int mode) {
     Team& t = C.t;
     const int nm = P.nm;
     if (mode == MODE_DIV) {
-        ROWS(p, P.nphi) P.pq[p] = (p < nm) ? row_div(P, P.idir[0], p) : 0.0;
+        ROWS(p, t.sm->phi, P.nphi) P.pq[p] = (p < nm) ? row_div(P, P.idir[0], p) : 0.0;
     } else if (mode == MODE_DIVT) {
-        ROWS(i, nm) {
+        ROWS(i, t.sm->nm, nm) {
             double t0, t1, t2;
             row_divT(P, P.pdir[0], i, t0, t1, t2);
             P.ihd[i] = t0;
@@ -1229,7 +1348,7 @@ __device__ bool ph_operator(Ctx& C, int mode) {
             P.ihd[2 * nm + i] = t2;
         }
     } else {
-        ROWS(i, nm) {
+        ROWS(i, t.sm->nm, nm) {
             double c0, c1, c2, a0, a1, a2;
             row_local(P, P.idir[0], i, c0, c1, c2, a0, a1, a2);
             P.ihd[i] = 2.0 * c0 + a0;
@@ -1254,7 +1373,7 @@ __device__ bool precond_solve(Ctx& C, int s) {
     // residual gr = H*0 + b with b = -g; preconditioned yv; direction -yv
     double acc[2] = {0.0, 0.0};
     double dummy[1] = {0.0};
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
         const double di = P.dinvA[i];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -1292,7 +1411,7 @@ __device__ bool precond_solve(Ctx& C, int s) {
         const double a = gy / dHd;
         const double* dv = P.idir[0];
         double a2[2] = {0.0, 0.0};
-        ROWS(i, nm) {
+        ROWS(i, t.sm->nm, nm) {
             const double di = P.dinvA[i];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -1332,7 +1451,7 @@ __device__ bool ph_hess32(Ctx& C, int s, const float* v, float beta, float* d, f
     const bool first = (beta == 0.0f);
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
         float c0, c1, c2;
         sell_dot3<8>(P.m_sptr, P.m_col, P.KA32, v, nm, i, c0, c1, c2);
         const float v0 = v[i], v1 = v[nm + i], v2 = v[2 * nm + i];
@@ -1382,7 +1501,7 @@ __device__ bool precond_solve32(Ctx& C, int s) {
     const double* g = P.GP[s];
     double acc[2] = {0.0, 0.0};
     double dummy[1] = {0.0};
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
         const float di = P.dinvA32[i];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -1419,7 +1538,7 @@ __device__ bool precond_solve32(Ctx& C, int s) {
         const double a = gy / dHd;
         const float af = (float)a;
         double a2[2] = {0.0, 0.0};
-        ROWS(i, nm) {
+        ROWS(i, t.sm->nm, nm) {
             const float di = P.dinvA32[i];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -1458,7 +1577,7 @@ __device__ bool ph_dir_dots(Ctx& C, int a, int c, double (&dots)[8]) {
     const double* go = P.GP[c];
     double dummy[1] = {0.0};
     for (int k = 0; k < 8; ++k) dots[k] = 0.0;
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
 #pragma unroll
         for (int q3 = 0; q3 < 3; ++q3) {
             const int q = q3 * nm + i;
@@ -1487,7 +1606,7 @@ __device__ bool ph_dir_write(Ctx& C, int a, int kind, double beta, double& dmax)
     const double b = (kind == 3) ? 0.0 : beta;   // b == 0: d_old is not read
     double mx[1] = {0.0};
     double dummy[1] = {0.0};
-    ROWS(i, nm) {
+    ROWS(i, t.sm->nm, nm) {
         double n2 = 0.0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -1660,8 +1779,11 @@ __device__ int minimize(Ctx& C, int& cur) {
 
 // The solver on one team of nb blocks (this block is number rank).
 __device__ __forceinline__ void solver_body(const Problem& P, int nb, int rank) {
+    __shared__ TeamSmem team_smem;
     Ctx C;
     C.P = &P;
+    C.t.sm = &team_smem;
+    C.t.target = 0;
     C.t.nb = nb;
     C.t.rank = rank;
     C.t.count = reinterpret_cast<unsigned long long*>(P.bar);
@@ -1669,6 +1791,20 @@ __device__ __forceinline__ void solver_body(const Problem& P, int nb, int rank) 
     C.t.part = P.partials;
     C.t.epoch = 0;
     C.t.dead = false;
+    if (threadIdx.x == 0) {
+        TeamSmem& sm = team_smem;
+        sm.dead = 0;
+        sm.phi = make_share(C.t, (P.nphi + 31) >> 5);
+        sm.nm = make_share(C.t, (P.nm + 31) >> 5);
+        sm.phi4 = make_share(C.t, ((P.nphi >> 2) + 31) >> 5);
+        for (int l = 0; l < P.nlev; ++l) {
+            const int rpw = 32 / restrict_group(P, C.t, l);
+            sm.rows[l] = make_share(C.t, (P.lev[l].n + 31) >> 5);
+            sm.coarse[l] = make_share(C.t, (P.lev[l].nc + rpw - 1) / rpw);
+        }
+        sm.dense = make_share(C.t, P.nco);
+    }
+    __syncthreads();
     C.evals = C.nli = C.li = C.mi = C.ls_extra = C.mr = 0;
     C.li2 = C.li2_first = C.restarts = C.steepest = 0;
     C.y_is_g = 0;
@@ -1734,11 +1870,15 @@ __device__ __forceinline__ void solver_body(const Problem& P, int nb, int rank) 
     }
 }
 
-// One instantiation per occupancy target (minimum resident blocks per SM),
-// each compiled in its own translation unit (mm_kern_*.cu); the host picks
-// one through solver_kernel() / solver_batch_kernel().
+// One instantiation per occupancy target (MINB x 256 resident threads per
+// SM), each compiled in its own translation unit (mm_kern_*.cu); the host
+// picks one through solver_kernel() / solver_batch_kernel().  The single form
+// runs them as one block per SM (MM_BLOCK = MINB x 256, set by its unit): a
+// barrier of 152 blocks costs 1.25 us where one of 304 costs 1.42 us and one
+// of 608 2.28 us, and a reduction folds 152 partials.  Batches keep blocks of
+// 256 threads, so that small members can have a fraction of an SM.
 template <int MINB>
-__global__ void __launch_bounds__(MM_BLOCK, MINB) k_solver(const __grid_constant__ Problem P) {
+__global__ void __launch_bounds__(MM_BLOCK, MINB * 256 / MM_BLOCK) k_solver(const __grid_constant__ Problem P) {
     solver_body(P, (int)gridDim.x, (int)blockIdx.x);
 }
 
