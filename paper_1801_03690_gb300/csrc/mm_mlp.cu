@@ -4,11 +4,10 @@
 // of the scalar potential.  Plain NCG then runs to t1-t3 from the corrected
 // state, so the network only changes where the minimiser starts.
 //
-// The forward pass and the weight gradients run on the 5th-generation
-// tensor cores (tcgen05.mma, accumulators in tensor memory: mm_mlp_tc.cuh);
-// the same network on the warp-level mma.sync m16n8k16 path (BF16 operands,
-// FP32 accumulation) is kept as a measured comparison
-// (mm_mlp_set_tensor_path), and the activation-gradient kernel uses it:
+// The forward pass and the training pass run on the 5th-generation tensor
+// cores (tcgen05.mma, accumulators in tensor memory: mm_mlp_tc.cuh).  The same
+// network on the warp-level mma.sync m16n8k16 path (BF16 operands, FP32
+// accumulation) is kept as a measured comparison (mm_mlp_set_tensor_path):
 //   k_mlp_forward   persistent; the weights (BF16, [out][in]) live in shared
 //                   memory; inputs are standardised in FP32 (the network's
 //                   own mean and 1/std) before the BF16 conversion, then each
@@ -20,8 +19,8 @@
 //                   storing every dZ_l
 //   k_mlp_wgrad     split-K GEMM dW_l = dZ_l^T A_{l-1} over row chunks,
 //                   partial tiles to global memory, then k_mlp_wreduce sums
-//                   the partials in a fixed order (deterministic) and the
-//                   bias gradients
+//                   the partials in a fixed order (deterministic) and
+//                   k_mlp_bgrad the bias gradients
 //   k_mlp_adam      Adam on FP32 master weights, refreshes the BF16 copies
 // Fragment layouts follow the PTX ISA description of mma.m16n8k16 (.bf16):
 // with g = lane/4 and q = lane%4, A holds (g, 2q..2q+1), (g+8, 2q..), (g, 2q+8..),
@@ -406,34 +405,84 @@ __global__ void k_mlp_bgrad(long long n, int nout, const __nv_bfloat16* __restri
     if (threadIdx.x == 0) gb[o] = sh[0];
 }
 
-__global__ void k_mlp_loss(long long n, const float* __restrict__ Y, const float* __restrict__ T, float* out) {
-    __shared__ float sh[256];
+// The loss in two fixed-order stages that both tensor paths share, so that
+// equal outputs give an equal loss: the squared errors of a tile of 128 rows
+// in FP32, the tiles in FP64.
+__device__ __forceinline__ float row_loss(const float (&y)[NOUT], const float (&t)[NOUT]) {
     float s = 0.0f;
-    for (long long i = threadIdx.x; i < n * NOUT; i += blockDim.x) {
-        const float d = Y[i] - T[i];
-        s += d * d;
+#pragma unroll
+    for (int c = 0; c < NOUT; ++c) {
+        const float d = __fsub_rn(y[c], t[c]);
+        s = __fmaf_rn(d, d, s);
     }
+    return s;
+}
+
+// Sum of a tile's row losses, the first 128 threads of the block taking part
+// with one row each; the result is thread 0's.
+__device__ __forceinline__ float tile_loss(float v, float (&sh)[4]) {
+    const int t = threadIdx.x;
+    if (t < 128) {
+        for (int o = 16; o > 0; o >>= 1) v = __fadd_rn(v, __shfl_down_sync(0xffffffffu, v, o));
+        if ((t & 31) == 0) sh[t >> 5] = v;
+    }
+    __syncthreads();
+    return __fadd_rn(__fadd_rn(sh[0], sh[1]), __fadd_rn(sh[2], sh[3]));
+}
+
+__global__ void __launch_bounds__(128) k_mlp_tile_loss(long long n, const float* __restrict__ Y,
+                                                       const float* __restrict__ T, float* __restrict__ tiles) {
+    __shared__ float sh[4];
+    const long long r = (long long)blockIdx.x * 128 + threadIdx.x;
+    float y[NOUT], t[NOUT];
+#pragma unroll
+    for (int c = 0; c < NOUT; ++c) {
+        y[c] = r < n ? Y[r * NOUT + c] : 0.0f;
+        t[c] = r < n ? T[r * NOUT + c] : 0.0f;
+    }
+    const float v = tile_loss(row_loss(y, t), sh);
+    if (threadIdx.x == 0) tiles[blockIdx.x] = v;
+}
+
+// Mean over the tiles' losses by one block of 256 threads.
+__device__ __forceinline__ void fold_loss(long long n, const float* __restrict__ tiles, float* out) {
+    __shared__ double sh[256];
+    const long long nt = (n + 127) / 128;
+    double s = 0.0;
+    for (long long i = threadIdx.x; i < nt; i += 256) s += (double)tiles[i];
     sh[threadIdx.x] = s;
     __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+    for (int w = 128; w > 0; w >>= 1) {
         if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = sh[0] / ((float)n * NOUT);
+    if (threadIdx.x == 0) *out = (float)(sh[0] / ((double)n * NOUT));
 }
 
-__global__ void k_mlp_adam(int np, float* p, const float* g, float* m, float* v, __nv_bfloat16* wb, float lr,
-                           float b1, float b2, float eps, float c1, float c2) {
+__global__ void __launch_bounds__(256) k_mlp_loss(long long n, const float* __restrict__ tiles, float* out) {
+    fold_loss(n, tiles, out);
+}
+
+// Adam on the FP32 master weights; refreshes the BF16 copies.
+struct Adam {
+    float *p, *m, *v;
+    __nv_bfloat16* wb;
+    float lr, b1, b2, eps, c1, c2;
+};
+
+__device__ __forceinline__ void adam_update(const Adam& a, int i, float gi) {
+    const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * gi;
+    const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * gi * gi;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float w = a.p[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    a.p[i] = w;
+    a.wb[i] = __float2bfloat16(w);
+}
+
+__global__ void k_mlp_adam(int np, const float* g, const Adam a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float w = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    p[i] = w;
-    wb[i] = __float2bfloat16(w);
+    if (i < np) adam_update(a, i, g[i]);
 }
 
 __global__ void k_to_bf16(int n, const float* a, __nv_bfloat16* b) {
@@ -630,15 +679,18 @@ struct mm_mlp {
     __nv_bfloat16 *DZ1 = nullptr, *DZ2 = nullptr, *DZ3 = nullptr, *DZ4 = nullptr;
     float* Yb = nullptr;
     float* part = nullptr;
-    float* loss = nullptr;
+    float* tpart = nullptr;       // tcgen05 training path: partial gradients, one set per CTA
+    long long tcap = 0;
+    float* tiles = nullptr;       // squared errors of every 128 rows
+    float* loss = nullptr;        // the loss, and after it the error flag
     cudaStream_t stream = nullptr;
     // inference buffers for the warm start
     long long fcap = 0;
     float *F = nullptr, *FY = nullptr;
     mm::Problem* d_prob = nullptr;
     unsigned* d_max = nullptr;
-    int* d_err = nullptr;         // set by a tensor-core wait that ran out
-    int path = 0;                 // 0: tcgen05 forward pass, 1: mma.sync (comparison)
+    int* d_err = nullptr;         // set by a tensor-core wait that ran out (in loss[1])
+    int path = 0;                 // 0: tcgen05, 1: mma.sync (comparison)
 };
 
 namespace {
@@ -655,18 +707,15 @@ size_t fwd_smem() { return sizeof(FwdSmem); }
 size_t bwd_smem() { return sizeof(BwdSmem); }
 size_t wgrad_smem() { return (size_t)2 * KCH * (128 + 8) * sizeof(__nv_bfloat16); }
 
+// Work space of the mma.sync training path.
 int ensure(mm_mlp* M, long long n) {
     if (n <= M->cap) return MM_OK;
-    cudaFree(M->X0);
-    cudaFree(M->A1);
-    cudaFree(M->A2);
-    cudaFree(M->A3);
-    cudaFree(M->DZ1);
-    cudaFree(M->DZ2);
-    cudaFree(M->DZ3);
-    cudaFree(M->DZ4);
-    cudaFree(M->Yb);
-    cudaFree(M->part);
+    M->cap = 0;
+    for (void** q : {(void**)&M->X0, (void**)&M->A1, (void**)&M->A2, (void**)&M->A3, (void**)&M->DZ1, (void**)&M->DZ2,
+                     (void**)&M->DZ3, (void**)&M->DZ4, (void**)&M->Yb, (void**)&M->part}) {
+        cudaFree(*q);
+        *q = nullptr;
+    }
     const long long nch = (n + KCH - 1) / KCH;
     if (cudaMalloc(&M->X0, n * NIN * sizeof(__nv_bfloat16)) != cudaSuccess ||
         cudaMalloc(&M->A1, n * NH * sizeof(__nv_bfloat16)) != cudaSuccess ||
@@ -679,36 +728,54 @@ int ensure(mm_mlp* M, long long n) {
         cudaMalloc(&M->Yb, n * NOUT * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->part, (size_t)nch * NH * NH * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
-        M->cap = 0;
         return MM_ERR_OOM;
     }
     M->cap = n;
     return MM_OK;
 }
 
-int launch_forward(mm_mlp* M, const float* X, long long n, float* Y, bool train) {
+// Work space of the tcgen05 training path (one set of partials per CTA) and
+// the tiles' losses of both paths.
+int ensure_tiles(mm_mlp* M, long long n) {
+    if (!M->tpart && cudaMalloc(&M->tpart, (size_t)M->nsm * tc::PSTRIDE * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        M->tpart = nullptr;
+        return MM_ERR_OOM;
+    }
+    const long long nt = (n + tc::TM - 1) / tc::TM;
+    if (nt <= M->tcap) return MM_OK;
+    M->tcap = 0;
+    cudaFree(M->tiles);
+    M->tiles = nullptr;
+    if (cudaMalloc(&M->tiles, nt * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        return MM_ERR_OOM;
+    }
+    M->tcap = nt;
+    return MM_OK;
+}
+
+int launch_forward(mm_mlp* M, const float* X, long long n, float* Y) {
     if (M->path == 0) {
         const int grid = std::max(1, std::min((int)((n + tc::TM - 1) / tc::TM), 2 * M->nsm));
-        tc::k_mlp_forward_tc<<<grid, tc::TM, sizeof(tc::Smem), M->stream>>>(
-            n, X, M->wb, M->p, M->norm, Y, train ? M->A1 : nullptr, train ? M->A2 : nullptr,
-            train ? M->A3 : nullptr, train ? M->X0 : nullptr, M->d_err);
+        tc::k_mlp_forward_tc<<<grid, tc::TM, sizeof(tc::Smem), M->stream>>>(n, X, M->wb, M->p, M->norm, Y, M->d_err);
         MK(cudaGetLastError());
         return MM_OK;
     }
     const int grid = std::max(1, std::min((int)((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK), 2 * M->nsm));
-    k_mlp_forward<<<grid, WARPS * 32, fwd_smem(), M->stream>>>(n, X, M->wb, M->p, M->norm, Y, train ? M->A1 : nullptr,
-                                                               train ? M->A2 : nullptr, train ? M->A3 : nullptr,
-                                                               train ? M->X0 : nullptr);
+    k_mlp_forward<<<grid, WARPS * 32, fwd_smem(), M->stream>>>(n, X, M->wb, M->p, M->norm, Y, nullptr, nullptr, nullptr,
+                                                               nullptr);
     MK(cudaGetLastError());
     return MM_OK;
 }
 
-// forward + backward into M->g (no update)
-int gradient(mm_mlp* M, const float* X, const float* T, long long n) {
+// forward + backward into M->g and the loss, on the mma.sync path
+int gradient_mma_sync(mm_mlp* M, const float* X, const float* T, long long n) {
     int rc;
     if ((rc = ensure(M, n))) return rc;
-    if ((rc = launch_forward(M, X, n, M->Yb, true))) return rc;
     const int grid = std::max(1, std::min((int)((n + ROWS_PER_BLOCK - 1) / ROWS_PER_BLOCK), 2 * M->nsm));
+    k_mlp_forward<<<grid, WARPS * 32, fwd_smem(), M->stream>>>(n, X, M->wb, M->p, M->norm, M->Yb, M->A1, M->A2, M->A3,
+                                                               M->X0);
     k_mlp_backward<<<grid, WARPS * 32, bwd_smem(), M->stream>>>(n, M->Yb, T, M->wb, M->A1, M->A2, M->A3, M->DZ4,
                                                                 M->DZ3, M->DZ2, M->DZ1);
     MK(cudaGetLastError());
@@ -721,15 +788,38 @@ int gradient(mm_mlp* M, const float* X, const float* T, long long n) {
                    {NH, NH, OFF_W3, OFF_B3, M->DZ3, M->A2},
                    {NOUT, NH, OFF_W4, OFF_B4, M->DZ4, M->A3}};
     for (auto& l : layers) {
-        if (M->path == 0)
-            tc::k_mlp_wgrad_tc<<<nch, tc::TM, sizeof(tc::WgSmem), M->stream>>>(n, l.nout, l.nin, l.dz, l.a, M->part,
-                                                                              M->d_err);
-        else
-            k_mlp_wgrad<<<nch, WARPS * 32, wgrad_smem(), M->stream>>>(n, l.nout, l.nin, l.dz, l.a, M->part);
+        k_mlp_wgrad<<<nch, WARPS * 32, wgrad_smem(), M->stream>>>(n, l.nout, l.nin, l.dz, l.a, M->part);
         MK(cudaGetLastError());
         const int nw = l.nout * l.nin;
         k_mlp_wreduce<<<(nw + 255) / 256, 256, 0, M->stream>>>(nch, nw, M->part, M->g + l.offw);
         k_mlp_bgrad<<<l.nout, 256, 0, M->stream>>>(n, l.nout, l.dz, M->g + l.offb);
+        MK(cudaGetLastError());
+    }
+    k_mlp_tile_loss<<<(unsigned)((n + 127) / 128), 128, 0, M->stream>>>(n, M->Yb, T, M->tiles);
+    k_mlp_loss<<<1, 256, 0, M->stream>>>(n, M->tiles, M->loss);
+    MK(cudaGetLastError());
+    return MM_OK;
+}
+
+// Gradients into M->g and the loss into M->loss; adam != nullptr: the update
+// follows.
+int gradient(mm_mlp* M, const float* X, const float* T, long long n, const Adam* adam) {
+    int rc;
+    if ((rc = ensure_tiles(M, n))) return rc;
+    if (M->path == 0) {
+        const int grid = (int)std::min((n + tc::TM - 1) / tc::TM, (long long)M->nsm);
+        const int vec = (reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(T)) % 16 == 0;
+        tc::k_mlp_train_tc<<<grid, tc::TT, sizeof(tc::TrainSmem), M->stream>>>(n, X, T, vec, M->wb, M->p, M->norm,
+                                                                             M->tpart, M->tiles, M->d_err);
+        MK(cudaGetLastError());
+        tc::k_mlp_reduce<<<(NPARAM + 63) / 64 + 1, 256, 0, M->stream>>>(n, grid, M->tpart, M->tiles, M->g, M->loss,
+                                                                       adam != nullptr, adam ? *adam : Adam{});
+        MK(cudaGetLastError());
+        return MM_OK;
+    }
+    if ((rc = gradient_mma_sync(M, X, T, n))) return rc;
+    if (adam) {
+        k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, M->stream>>>(NPARAM, M->g, *adam);
         MK(cudaGetLastError());
     }
     return MM_OK;
@@ -743,6 +833,20 @@ int check_err(mm_mlp* M) {
     if (!e) return MM_OK;
     MK(cudaMemset(M->d_err, 0, sizeof(int)));
     return MM_ERR_DEVICE_TIMEOUT;
+}
+
+// Wait for the stream; the last pass's loss, and check_err's status from the
+// same copy (the flag is the word after the loss).
+int read_loss(mm_mlp* M, float* loss) {
+    struct {
+        float loss;
+        int err;
+    } h;
+    MK(cudaMemcpyAsync(&h, M->loss, sizeof(h), cudaMemcpyDeviceToHost, M->stream));
+    MK(cudaStreamSynchronize(M->stream));
+    if (h.err) return check_err(M);
+    *loss = h.loss;
+    return MM_OK;
 }
 
 }  // namespace
@@ -776,10 +880,12 @@ int mm_mlp_create(mm_mlp** out, int device, uint64_t seed) {
         cudaMalloc(&M->g, NPARAM * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->am, NPARAM * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->av, NPARAM * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&M->loss, sizeof(float)) != cudaSuccess || cudaMalloc(&M->d_prob, sizeof(mm::Problem)) != cudaSuccess ||
+        cudaMalloc(&M->loss, 2 * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&M->d_prob, sizeof(mm::Problem)) != cudaSuccess ||
         cudaMalloc(&M->norm, 2 * NIN * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&M->d_max, sizeof(unsigned)) != cudaSuccess || cudaMalloc(&M->d_err, sizeof(int)) != cudaSuccess)
+        cudaMalloc(&M->d_max, sizeof(unsigned)) != cudaSuccess)
         return bail(MM_ERR_OOM);
+    M->d_err = reinterpret_cast<int*>(M->loss + 1);
     if (cudaMemset(M->d_err, 0, sizeof(int)) != cudaSuccess) return bail(MM_ERR_CUDA);
     {
         float id[2 * NIN];
@@ -799,8 +905,8 @@ int mm_mlp_create(mm_mlp** out, int device, uint64_t seed) {
                              (int)sizeof(tc::Smem)) != cudaSuccess ||
         cudaFuncSetAttribute(tc::k_mlp_forward_tc, cudaFuncAttributePreferredSharedMemoryCarveout, 100) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(tc::k_mlp_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(tc::WgSmem)) != cudaSuccess)
+        cudaFuncSetAttribute(tc::k_mlp_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(tc::TrainSmem)) != cudaSuccess)
         return bail(MM_ERR_CUDA);
     // He-uniform initialisation (host RNG, seeded), zero biases
     std::vector<float> h(NPARAM, 0.0f);
@@ -824,7 +930,7 @@ void mm_mlp_destroy(mm_mlp* M) {
     for (void* q : {(void*)M->p, (void*)M->norm, (void*)M->wb, (void*)M->g, (void*)M->am, (void*)M->av, (void*)M->loss,
                     (void*)M->X0, (void*)M->A1, (void*)M->A2, (void*)M->A3, (void*)M->DZ1, (void*)M->DZ2,
                     (void*)M->DZ3, (void*)M->DZ4, (void*)M->Yb, (void*)M->part, (void*)M->F, (void*)M->FY,
-                    (void*)M->d_prob, (void*)M->d_max, (void*)M->d_err})
+                    (void*)M->d_prob, (void*)M->d_max, (void*)M->tpart, (void*)M->tiles})
         if (q) cudaFree(q);
     if (M->stream) cudaStreamDestroy(M->stream);
     delete M;
@@ -867,7 +973,7 @@ int mm_mlp_get_params(mm_mlp* M, float* params, int64_t count) {
 int mm_mlp_forward(mm_mlp* M, const float* X_dev, int64_t n, float* Y_dev) {
     if (!M || !X_dev || !Y_dev || n < 1) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    int rc = launch_forward(M, X_dev, n, Y_dev, false);
+    int rc = launch_forward(M, X_dev, n, Y_dev);
     if (rc) return rc;
     MK(cudaStreamSynchronize(M->stream));
     return check_err(M);
@@ -877,36 +983,25 @@ int mm_mlp_gradient(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t n
                     float* loss_out) {
     if (!M || !X_dev || !T_dev || n < 1) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    int rc = gradient(M, X_dev, T_dev, n);
+    int rc = gradient(M, X_dev, T_dev, n, nullptr);
     if (rc) return rc;
-    k_mlp_loss<<<1, 256, 0, M->stream>>>(n, M->Yb, T_dev, M->loss);
-    MK(cudaGetLastError());
-    MK(cudaStreamSynchronize(M->stream));
-    if ((rc = check_err(M))) return rc;
+    float loss = 0.0f;
+    if ((rc = read_loss(M, &loss))) return rc;
     if (grad_host) MK(cudaMemcpy(grad_host, M->g, NPARAM * sizeof(float), cudaMemcpyDeviceToHost));
-    if (loss_out) MK(cudaMemcpy(loss_out, M->loss, sizeof(float), cudaMemcpyDeviceToHost));
+    if (loss_out) *loss_out = loss;
     return MM_OK;
 }
 
 int mm_mlp_train_step(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t n, float lr, float* loss_out) {
     if (!M || !X_dev || !T_dev || n < 1 || !(lr > 0.0f)) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    int rc = gradient(M, X_dev, T_dev, n);
+    const float b1 = 0.9f, b2 = 0.999f;
+    const float step = (float)(M->step + 1);
+    const Adam adam{M->p, M->am, M->av, M->wb, lr, b1, b2, 1e-8f, 1.0f - std::pow(b1, step), 1.0f - std::pow(b2, step)};
+    const int rc = gradient(M, X_dev, T_dev, n, &adam);
     if (rc) return rc;
     M->step++;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - std::pow(b1, (float)M->step), c2 = 1.0f - std::pow(b2, (float)M->step);
-    k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, M->stream>>>(NPARAM, M->p, M->g, M->am, M->av, M->wb, lr, b1, b2,
-                                                             1e-8f, c1, c2);
-    MK(cudaGetLastError());
-    if (loss_out) {
-        k_mlp_loss<<<1, 256, 0, M->stream>>>(n, M->Yb, T_dev, M->loss);
-        MK(cudaGetLastError());
-        MK(cudaMemcpyAsync(loss_out, M->loss, sizeof(float), cudaMemcpyDeviceToHost, M->stream));
-        MK(cudaStreamSynchronize(M->stream));
-        if ((rc = check_err(M))) return rc;
-    }
-    return MM_OK;
+    return loss_out ? read_loss(M, loss_out) : MM_OK;
 }
 
 }  // extern "C"
@@ -1074,7 +1169,7 @@ int mm_warmstart_apply(mm_ctx* ctx, mm_mlp* M, const double mu0h_next[3], double
     }
     int rc = mm_warmstart_features(ctx, mu0h_next, M->F);
     if (rc) return rc;
-    if ((rc = launch_forward(M, M->F, v.nm, M->FY, false))) return rc;
+    if ((rc = launch_forward(M, M->F, v.nm, M->FY))) return rc;
     MK(cudaStreamSynchronize(M->stream));
     if ((rc = check_err(M))) return mm::ctx_fail(ctx, rc, "a tensor-core wait of the network ran out");
     mm::DevState hs;

@@ -225,3 +225,30 @@ def test_tcgen05_weight_gradient_matches_mma_sync_and_reference(n):
                                  T.cpu().numpy().astype(np.float64), round_bf16=True)
     for (gw, gb), (rw, rb) in zip(_params_list(g_tc), gr):
         np.testing.assert_allclose(gw, rw, rtol=0, atol=3e-2 * np.abs(rw).max())
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128 + 1, 8 * 152 * 128 + 300])
+def test_training_pass_edges(n):
+    """The fused tcgen05 training pass at the edges of its tiles (128 rows), of
+    its grid (152 SMs) and of the tiles it accumulates before a flush (8), on
+    aligned and on odd addresses, against the mma.sync path: the same products
+    of the same BF16 values in FP32, summed in another order.  Rounding errors
+    of n / 128 partial sums of either sign grow like 2^-24 sqrt(n / 128) of the
+    largest partial: 2e-6 at the largest n, bound 1e-5."""
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    net = MLP(seed=6)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    buf = torch.randn(20 * n + 1, generator=g, device="cuda")
+    X, T = buf[:16 * n].view(n, 16), buf[16 * n:20 * n].view(n, 4)
+    g_tc, loss_tc = net.gradient(X, T)
+    odd = torch.cat([buf[:1], buf[:-1]])[1:]                        # the same values, 4 bytes off a 16-byte boundary
+    assert odd.data_ptr() % 16 == 4
+    g_odd, loss_odd = net.gradient(odd[:16 * n].view(n, 16), odd[16 * n:20 * n].view(n, 4))
+    assert loss_odd == loss_tc and np.array_equal(g_odd, g_tc)
+    net.set_tensor_path(1)
+    g_ms, loss_ms = net.gradient(X, T)
+    assert loss_tc == loss_ms
+    for (gw, gb), (rw, rb) in zip(_params_list(g_tc), _params_list(g_ms)):
+        assert np.abs(gw - rw).max() <= 1e-5 * np.abs(rw).max()
+        assert np.abs(gb - rb).max() <= 1e-5 * np.abs(rb).max()
