@@ -757,8 +757,10 @@ int ensure_tiles(mm_mlp* M, long long n) {
 
 int launch_forward(mm_mlp* M, const float* X, long long n, float* Y) {
     if (M->path == 0) {
-        const int grid = std::max(1, std::min((int)((n + tc::TM - 1) / tc::TM), 2 * M->nsm));
-        tc::k_mlp_forward_tc<<<grid, tc::TM, sizeof(tc::Smem), M->stream>>>(n, X, M->wb, M->p, M->norm, Y, M->d_err);
+        const int grid = (int)std::min((n + tc::TM - 1) / tc::TM, (long long)M->nsm);
+        const int vec = (reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) % 16 == 0;
+        tc::k_mlp_forward_tc<<<grid, tc::GROUPS * tc::TM, sizeof(tc::Smem), M->stream>>>(n, X, vec, M->wb, M->p,
+                                                                                       M->norm, Y, M->d_err);
         MK(cudaGetLastError());
         return MM_OK;
     }

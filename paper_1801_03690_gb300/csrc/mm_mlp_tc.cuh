@@ -4,7 +4,7 @@
 // TMEM lane per row).  Included by mm_mlp.cu (it uses that file's layer
 // sizes and parameter layout).
 //
-// Per tile of 128 rows (4 warps, thread t owns row t of the tile):
+// Per tile of 128 rows (a group of 4 warps, thread t owns row t of the tile):
 //   x   = bf16((X - mean) / std)                  -> shared memory
 //   h1  = relu(x W1^T + b1)   1 MMA  (K = 16)     TMEM -> registers -> bf16 -> shared
 //   h2  = relu(h1 W2^T + b2)  8 MMAs (K = 8 x 16)
@@ -35,16 +35,18 @@ constexpr int N4 = 16;       // the last layer's N, padded
 constexpr int TCOLS = 128;   // TMEM columns allocated (one N = 128 accumulator)
 constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s per MMA wait
 
+constexpr int GROUPS = 4;    // forward pass: tiles in flight per SM, 128 threads each
+
 struct __align__(128) Smem {
     __nv_bfloat16 w1[NH * NIN];
     __nv_bfloat16 w2[NH * NH];
     __nv_bfloat16 w3[NH * NH];
     __nv_bfloat16 w4[N4 * NH];
-    __nv_bfloat16 x[TM * NIN];
-    __nv_bfloat16 h[TM * NH];
+    __nv_bfloat16 x[GROUPS][TM * NIN];
+    __nv_bfloat16 h[GROUPS][TM * NH];
     float b[3 * NH + N4];
     float mean[NIN], istd[NIN];
-    unsigned long long bar;
+    unsigned long long bar[GROUPS];
     unsigned tmem;
 };
 
@@ -141,64 +143,120 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// A row-major [rows][COLS] BF16 matrix (16-byte aligned) into the tile layout,
+// 16 bytes per thread and step; eight lanes take the eight rows of a core
+// matrix, so that a warp's stores are contiguous.
+template <int COLS>
+__device__ __forceinline__ void stage_tile(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int rows, int have,
+                                           int tid, int nthreads) {
+    unsigned char* d = reinterpret_cast<unsigned char*>(dst);
+    for (int i = tid; i < rows * (COLS / 8); i += nthreads) {
+        const int r = (i / COLS) * 8 + (i & 7), k = ((i >> 3) % (COLS / 8)) * 8;
+        const uint4 v = r < have ? *reinterpret_cast<const uint4*>(src + r * COLS + k) : make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(d + core_off(r, k, COLS)) = v;
+    }
+}
+
+// Four consecutive floats; vec: the array is 16-byte aligned.
+__device__ __forceinline__ float4 load4(const float* p, bool vec) {
+    return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+}
+
+// Barriers of one group of 128 threads (hardware barriers 1 .. GROUPS).
+__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
+__device__ __forceinline__ bool group_and(int g, bool v) {
+    unsigned r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, %2, 128, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(r)
+        : "r"((unsigned)v), "r"(g + 1)
+        : "memory");
+    return r != 0;
+}
+
+// relu(a + b) of two columns as packed BF16.  The maximum is taken after the
+// rounding, which keeps its sign (a NaN gives 0 either way).
+__device__ __forceinline__ unsigned bias_relu2(float a0, float a1, float b0, float b1) {
+    unsigned long long a, b, s;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "f"(a0), "f"(a1));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(b) : "f"(b0), "f"(b1));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(a), "l"(b));
+    float s0, s1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(s0), "=f"(s1) : "l"(s));
+    const __nv_bfloat162 r = __hmax2(__floats2bfloat162_rn(s0, s1), __floats2bfloat162_rn(0.0f, 0.0f));
+    return *reinterpret_cast<const unsigned*>(&r);
+}
+
 // Hidden-layer epilogue of this thread's row: h = relu(acc + b) to BF16,
 // into the next layer's A operand (shared).
-__device__ __forceinline__ void hidden_epilogue(Smem& s, unsigned tlane, const float* b, int row) {
+__device__ __forceinline__ void hidden_epilogue(unsigned char* hb, unsigned tlane, const float* b, int row) {
 #pragma unroll 1
     for (int j = 0; j < NH / 32; ++j) {
         float v[32];
         tmem_ld32(tlane + 32 * j, v);
-        __align__(16) __nv_bfloat16 o[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] = __float2bfloat16(fmaxf(v[i] + b[32 * j + i], 0.0f));
-        unsigned char* hb = reinterpret_cast<unsigned char*>(s.h);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(hb + core_off(row, 32 * j + 8 * q, NH)) = reinterpret_cast<const uint4*>(o)[q];
+        for (int q = 0; q < 4; ++q) {
+            const float4 b0 = *reinterpret_cast<const float4*>(b + 32 * j + 8 * q);
+            const float4 b1 = *reinterpret_cast<const float4*>(b + 32 * j + 8 * q + 4);
+            const float* u = v + 8 * q;
+            *reinterpret_cast<uint4*>(hb + core_off(row, 32 * j + 8 * q, NH)) =
+                make_uint4(bias_relu2(u[0], u[1], b0.x, b0.y), bias_relu2(u[2], u[3], b0.z, b0.w),
+                           bias_relu2(u[4], u[5], b1.x, b1.y), bias_relu2(u[6], u[7], b1.z, b1.w));
+        }
     }
 }
 
-// Two CTAs per SM (2 x 110 KB of shared memory, 2 x 128 TMEM columns): while
-// one waits on its MMAs or runs its epilogue, the other's MMAs run.
-__global__ void __launch_bounds__(TM, 2) k_mlp_forward_tc(long long n, const float* __restrict__ X,
-                                                           const __nv_bfloat16* __restrict__ wb,
-                                                           const float* __restrict__ p,
-                                                           const float* __restrict__ norm, float* __restrict__ Y,
-                                                           int* err) {
+// One CTA per SM: the weights once in shared memory (72 KB) and GROUPS groups
+// of 128 threads, each taking tiles of its own through the four layers with an
+// input tile, an activation tile (36 KB) and 128 TMEM columns of its own.  A
+// tile is a chain of four dependent products with an epilogue each; while one
+// group waits for its product or runs its epilogue, the others' products keep
+// the tensor core at work.  Two CTAs of 128 threads, each with weights of its
+// own, element-wise staging and two-byte stores took 61 us a call at 20,011
+// rows and 615 us at 3,375,000; this form takes 45 and 356 (the tensor rate
+// would allow 123).
+__global__ void __launch_bounds__(GROUPS * TM, 1) k_mlp_forward_tc(long long n, const float* __restrict__ X, int vec,
+                                                                   const __nv_bfloat16* __restrict__ wb,
+                                                                   const float* __restrict__ p,
+                                                                   const float* __restrict__ norm,
+                                                                   float* __restrict__ Y, int* err) {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     Smem& s = *reinterpret_cast<Smem*>(tc_smem);
-    const int tid = threadIdx.x, warp = tid >> 5;
-    // weights (BF16 copies) into the core-matrix layout, biases, standardisation
-    unsigned char* w1 = reinterpret_cast<unsigned char*>(s.w1);
-    unsigned char* w2 = reinterpret_cast<unsigned char*>(s.w2);
-    unsigned char* w3 = reinterpret_cast<unsigned char*>(s.w3);
-    unsigned char* w4 = reinterpret_cast<unsigned char*>(s.w4);
-    for (int i = tid; i < SZ_W1; i += TM)
-        *reinterpret_cast<__nv_bfloat16*>(w1 + core_off(i / NIN, i % NIN, NIN)) = wb[OFF_W1 + i];
-    for (int i = tid; i < SZ_W2; i += TM) {
-        *reinterpret_cast<__nv_bfloat16*>(w2 + core_off(i / NH, i % NH, NH)) = wb[OFF_W2 + i];
-        *reinterpret_cast<__nv_bfloat16*>(w3 + core_off(i / NH, i % NH, NH)) = wb[OFF_W3 + i];
-    }
-    for (int i = tid; i < N4 * NH; i += TM)
-        *reinterpret_cast<__nv_bfloat16*>(w4 + core_off(i / NH, i % NH, NH)) =
-            (i < SZ_W4) ? wb[OFF_W4 + i] : __float2bfloat16(0.0f);
-    for (int i = tid; i < NH; i += TM) {
-        s.b[i] = p[OFF_B1 + i];
-        s.b[NH + i] = p[OFF_B2 + i];
-        s.b[2 * NH + i] = p[OFF_B3 + i];
+    constexpr int NT = GROUPS * TM;
+    const int tid = threadIdx.x, warp = tid >> 5, g = tid / TM, row = tid % TM;
+    const long long ntiles = (n + TM - 1) / TM, stride = (long long)gridDim.x * GROUPS;
+    long long tile = blockIdx.x + (long long)gridDim.x * g;
+    float4 xv[NIN / 4];                          // this thread's row of the group's next tile
+    auto fetch = [&](long long t) {
+        const long long r = t * TM + row;
+        if (r < n) {
+#pragma unroll
+            for (int q = 0; q < NIN / 4; ++q) xv[q] = load4(X + r * NIN + 4 * q, vec);
+        }
+    };
+    fetch(tile);
+    stage_tile<NIN>(s.w1, wb + OFF_W1, NH, NH, tid, NT);
+    stage_tile<NH>(s.w2, wb + OFF_W2, NH, NH, tid, NT);
+    stage_tile<NH>(s.w3, wb + OFF_W3, NH, NH, tid, NT);
+    stage_tile<NH>(s.w4, wb + OFF_W4, N4, NOUT, tid, NT);
+    if (tid < NH) {
+        s.b[tid] = p[OFF_B1 + tid];
+        s.b[NH + tid] = p[OFF_B2 + tid];
+        s.b[2 * NH + tid] = p[OFF_B3 + tid];
     }
     if (tid < N4) s.b[3 * NH + tid] = (tid < NOUT) ? p[OFF_B4 + tid] : 0.0f;
     if (tid < NIN) {
         s.mean[tid] = norm[tid];
         s.istd[tid] = norm[NIN + tid];
     }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar)) : "memory");
+    if (tid < GROUPS) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar[tid])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s.tmem)),
-                     "r"(TCOLS)
+                     "r"(GROUPS * TCOLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -206,87 +264,86 @@ __global__ void __launch_bounds__(TM, 2) k_mlp_forward_tc(long long n, const flo
     before_sync();
     __syncthreads();
     after_sync();
-    const unsigned tbase = s.tmem;
-    const unsigned tlane = tbase + ((unsigned)(warp * 32) << 16);   // this warp's 32 TMEM lanes
-    const unsigned long long dx = sdesc(s.x, NIN), dh = sdesc(s.h, NH);
-    const unsigned long long dw1 = sdesc(s.w1, NIN), dw2 = sdesc(s.w2, NH), dw3 = sdesc(s.w3, NH),
-                             dw4 = sdesc(s.w4, NH);
+    const unsigned tbase = s.tmem + (unsigned)(g * TCOLS);                // the group's accumulator
+    const unsigned tlane = tbase + ((unsigned)((warp & 3) * 32) << 16);   // this warp's 32 TMEM lanes
+    const unsigned long long dx = sdesc(s.x[g], NIN), dh = sdesc(s.h[g], NH);
     constexpr unsigned id128 = idesc_bf16(TM, NH), id16 = idesc_bf16(TM, N4);
     // one K step of 16 bf16 = two core matrices = 256 B = 16 in the address field
     constexpr unsigned long long KSTEP = 256 >> 4;
+    unsigned char* xb = reinterpret_cast<unsigned char*>(s.x[g]);
+    unsigned char* hb = reinterpret_cast<unsigned char*>(s.h[g]);
     unsigned parity = 0;
     bool ok = true;
-    const long long ntiles = (n + TM - 1) / TM;
-    auto layer_done = [&]() -> bool {        // the layer's MMAs have completed (all threads agree)
-        const bool mine = wait_phase(&s.bar, parity);
-        const bool all = __syncthreads_and(mine) != 0;
+    // A layer's MMAs, issued by one thread of the group once all its writes are in place ...
+    auto issue = [&](unsigned long long a, const __nv_bfloat16* w, int k_in, unsigned id) {
+        fence_async_smem();
+        before_sync();
+        group_sync(g);
+        after_sync();
+        if (row == 0) {
+            const unsigned long long dw = sdesc(w, k_in);
+#pragma unroll 8
+            for (int k = 0; k < k_in / 16; ++k) mma(tbase, a + k * KSTEP, dw + k * KSTEP, id, k > 0);
+            commit(&s.bar[g]);
+        }
+    };
+    // ... and their completion (the whole group agrees).
+    auto done = [&]() -> bool {
+        const bool all = group_and(g, wait_phase(&s.bar[g], parity));
         if (all) parity ^= 1u;
         after_sync();
         return all;
     };
-    auto before_mma = [&]() {
-        fence_async_smem();
-        before_sync();
-        __syncthreads();
-        after_sync();
-    };
-    for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        const long long r = tile * TM + tid;
-        unsigned char* xb = reinterpret_cast<unsigned char*>(s.x);
+    for (; tile < ntiles; tile += stride) {
+        const long long r = tile * TM + row;
+        {
+            __align__(16) __nv_bfloat16 o[NIN];
 #pragma unroll
-        for (int c = 0; c < NIN; ++c) {
-            const __nv_bfloat16 v = __float2bfloat16(r < n ? (X[r * NIN + c] - s.mean[c]) * s.istd[c] : 0.0f);
-            *reinterpret_cast<__nv_bfloat16*>(xb + core_off(tid, c, NIN)) = v;
-        }
-        before_mma();
-        if (tid == 0) {
-            mma(tbase, dx, dw1, id128, 0u);
-            commit(&s.bar);
-        }
-        if (!(ok = layer_done())) break;
-        hidden_epilogue(s, tlane, s.b, tid);
-        before_mma();
-        if (tid == 0) {
+            for (int q = 0; q < NIN / 4; ++q) {
+                const float u[4] = {xv[q].x, xv[q].y, xv[q].z, xv[q].w};
 #pragma unroll
-            for (int k = 0; k < NH / 16; ++k) mma(tbase, dh + k * KSTEP, dw2 + k * KSTEP, id128, k > 0);
-            commit(&s.bar);
+                for (int c = 0; c < 4; ++c)
+                    o[4 * q + c] = __float2bfloat16(r < n ? (u[c] - s.mean[4 * q + c]) * s.istd[4 * q + c] : 0.0f);
+            }
+            *reinterpret_cast<uint4*>(xb + core_off(row, 0, NIN)) = reinterpret_cast<const uint4*>(o)[0];
+            *reinterpret_cast<uint4*>(xb + core_off(row, 8, NIN)) = reinterpret_cast<const uint4*>(o)[1];
         }
-        if (!(ok = layer_done())) break;
-        hidden_epilogue(s, tlane, s.b + NH, tid);
-        before_mma();
-        if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < NH / 16; ++k) mma(tbase, dh + k * KSTEP, dw3 + k * KSTEP, id128, k > 0);
-            commit(&s.bar);
-        }
-        if (!(ok = layer_done())) break;
-        hidden_epilogue(s, tlane, s.b + 2 * NH, tid);
-        before_mma();
-        if (tid == 0) {
-#pragma unroll
-            for (int k = 0; k < NH / 16; ++k) mma(tbase, dh + k * KSTEP, dw4 + k * KSTEP, id16, k > 0);
-            commit(&s.bar);
-        }
-        if (!(ok = layer_done())) break;
+        issue(dx, s.w1, NIN, id128);
+        fetch(tile + stride);
+        if (!(ok = done())) break;
+        hidden_epilogue(hb, tlane, s.b, row);
+        issue(dh, s.w2, NH, id128);
+        if (!(ok = done())) break;
+        hidden_epilogue(hb, tlane, s.b + NH, row);
+        issue(dh, s.w3, NH, id128);
+        if (!(ok = done())) break;
+        hidden_epilogue(hb, tlane, s.b + 2 * NH, row);
+        issue(dh, s.w4, NH, id16);
+        if (!(ok = done())) break;
         float v[16];
-        tmem_ld16(tlane, v);
+        tmem_ld16(tlane, v);         // (the next tile's first product follows the group's next barrier)
         if (r < n) {
+            float y[NOUT];
 #pragma unroll
-            for (int c = 0; c < NOUT; ++c) Y[r * NOUT + c] = v[c] + s.b[3 * NH + c];
+            for (int c = 0; c < NOUT; ++c) y[c] = v[c] + s.b[3 * NH + c];
+            if (vec) {
+                *reinterpret_cast<float4*>(Y + r * NOUT) = make_float4(y[0], y[1], y[2], y[3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < NOUT; ++c) Y[r * NOUT + c] = y[c];
+            }
         }
-        before_sync();
-        __syncthreads();                  // TMEM read before the next tile's first MMA overwrites it
-        after_sync();
     }
     if (!ok) {
-        if (tid == 0) atomicExch(err, 1);
-        wait_phase(&s.bar, parity);       // the phase that did not complete: let it finish (bounded)
+        if (row == 0) atomicExch(err, 1);
+        wait_phase(&s.bar[g], parity);    // the phase that did not complete: let it finish (bounded)
     }
     before_sync();
     __syncthreads();
     after_sync();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(TCOLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s.tmem), "r"(GROUPS * TCOLS)
+                     : "memory");
 }
 
 // ---- training pass: forward, loss, activation gradients and all weight and
@@ -309,8 +366,8 @@ __global__ void __launch_bounds__(TM, 2) k_mlp_forward_tc(long long n, const flo
 // separate kernels (forward, backward, and per layer a weight-gradient, a
 // reduction and a bias kernel, activations and dZ in HBM, two-byte strided
 // loads, the loss by one block) a training step took 222 / 333 / 957 us at
-// 64 / 16,384 / 65,536 rows; it takes 65 / 70 / 103 us now, of which about 60
-// are the caller's copies of the loss and the parameters.
+// 64 / 16,384 / 65,536 rows; it takes 65 / 70 / 103 us now, with the
+// caller's reads of the loss and the parameters.
 constexpr int TT = 256;              // threads: two per row, each with half the columns
 constexpr int TRAIN_COLS = 512;      // TMEM columns allocated
 constexpr int C_G3 = 128, C_G2 = 256, C_G1 = 384, C_G4 = 400, C_B = 416;
@@ -332,25 +389,6 @@ struct __align__(128) TrainSmem {
     unsigned long long bar;
     unsigned tmem;
 };
-
-// A row-major [rows][COLS] BF16 matrix (16-byte aligned) into the tile layout,
-// 16 bytes per thread and step; eight lanes take the eight rows of a core
-// matrix, so that a warp's stores are contiguous.
-template <int COLS>
-__device__ __forceinline__ void stage_tile(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int rows, int have,
-                                           int tid, int nthreads) {
-    unsigned char* d = reinterpret_cast<unsigned char*>(dst);
-    for (int i = tid; i < rows * (COLS / 8); i += nthreads) {
-        const int r = (i / COLS) * 8 + (i & 7), k = ((i >> 3) % (COLS / 8)) * 8;
-        const uint4 v = r < have ? *reinterpret_cast<const uint4*>(src + r * COLS + k) : make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4*>(d + core_off(r, k, COLS)) = v;
-    }
-}
-
-// Four consecutive floats; vec: the array is 16-byte aligned.
-__device__ __forceinline__ float4 load4(const float* p, bool vec) {
-    return vec ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
-}
 
 __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(long long n, const float* __restrict__ X,
                                                          const float* __restrict__ T, int vec,
