@@ -252,3 +252,39 @@ def test_training_pass_edges(n):
     for (gw, gb), (rw, rb) in zip(_params_list(g_tc), _params_list(g_ms)):
         assert np.abs(gw - rw).max() <= 1e-5 * np.abs(rw).max()
         assert np.abs(gb - rb).max() <= 1e-5 * np.abs(rb).max()
+
+
+@pytest.mark.parametrize("n,centre,scale", [(2, 0.0, 1.0), (127, 3.0, 0.5), (128 * 33 + 5, 1e4, 1.0), (700001, -2.0, 3.0),
+                                            (1000, 1e22, 1e21), (5000, 1e-30, 1e-30)])
+def test_statistics_edges(n, centre, scale):
+    """The one-pass statistics against FP64 ones of the same values: tails of a
+    block and of a fold, means far from zero, an odd address, and squares
+    beyond or below FP32, which go to (or give the same as) the FP64 passes.
+    Means and scales come back as FP32 (relative error 2^-24, bound 1e-6 of the
+    deviation or of the value); the target scales as FP64 from sums of pairs of
+    FP32 words (2^-45 at worst, bound 1e-12)."""
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    net = MLP(seed=1)
+    rng = np.random.default_rng(n)
+    buf = (centre + scale * rng.normal(size=20 * n + 1)).astype(np.float32)
+    X = buf[1:16 * n + 1].reshape(n, 16)
+    X[:, 13] = 0.37                                          # a constant column
+    T = buf[16 * n + 1:].reshape(n, 4)
+    dev = torch.tensor(buf, device="cuda")
+    Xd, Td = dev[1:16 * n + 1].view(n, 16), dev[16 * n + 1:].view(n, 4)
+    net.fit_input_norm(Xd)
+    mean, istd = net.input_norm()
+    X64, T64 = X.astype(np.float64), T.astype(np.float64)
+    m, s = X64.mean(0), X64.std(0, ddof=1)
+    s = np.where(s > 1e-6 * (np.abs(m) + 1.0), s, 1.0)
+    np.testing.assert_allclose(mean, m, rtol=1e-6, atol=1e-6 * X64.std(0, ddof=1).max())
+    np.testing.assert_allclose(istd, 1.0 / s, rtol=1e-6)
+    Tn, sm, sp = net.fit_target_scales(Td)
+    em, ep = max(T64[:, :3].std(ddof=1), 1e-12), max(T64[:, 3].std(ddof=1), 1e-12)
+    assert abs(sm - em) <= 1e-12 * em and abs(sp - ep) <= 1e-12 * ep
+    ref = T / np.array([sm, sm, sm, sp], dtype=np.float32)
+    np.testing.assert_allclose(Tn.cpu().numpy(), ref, rtol=2.0 ** -22)
+    Xd[n - 1, 3] = float("nan")
+    with pytest.raises(Exception):
+        net.fit_input_norm(Xd)
