@@ -37,7 +37,22 @@ struct Share {
     int full, tail, count;
 };
 
+// Scalars of the running CG solve (Algorithm 1), kept by the lanes that fold
+// the team's values.  Each is one lane's work: an FP64 instruction of every
+// warp occupies the SM's FP64 pipe for 19 cycles a warp, so that a division
+// evaluated by all 16 (32) warps of a block took about 2 (4) us on the chain of
+// every CG step, twice.
+struct CgScalars {
+    double rz, rz_old;               // r.z, and before the last step
+    double a, beta;                  // step length, beta
+    double rmax;                     // FP32 solve: largest |r|^2 since the last update
+    float af, betaf;
+    double eps;                      // preconditioner solve: limit of |r| (li3)
+    int stop;                        // the residual meets the solve's (or the update's) limit
+};
+
 struct TeamSmem {
+    CgScalars cg;
     double v[kFlat][MM_BLOCK];       // one value per thread
     double w[MM_MAXRED][kWarps];     // one value per warp
     double res[MM_MAXRED];           // the team's values
@@ -165,9 +180,13 @@ __device__ __forceinline__ double warp_sums_shared(double (&v)[KP]) {
 // Second half of a team reduction: the block's partial values of K
 // quantities (the first NS sums, the others maxima) are in `part`; after the
 // barrier every block folds all partials identically, one warp per quantity,
-// into t.sm->res.
-template <int K, int NS>
-__device__ __forceinline__ bool team_combine(Team& t, const double* part) {
+// into t.sm->res.  fin(k, value) runs on the lane that folded value k; what it
+// writes to shared memory every thread may read afterwards.
+struct NoFinish {
+    __device__ void operator()(int, double) const {}
+};
+template <int K, int NS, class Fin>
+__device__ __forceinline__ bool team_combine(Team& t, const double* part, Fin fin) {
     if (!team_sync(t)) return false;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = warp; k < K; k += kWarps) {
@@ -185,7 +204,10 @@ __device__ __forceinline__ bool team_combine(Team& t, const double* part) {
             s = j0 == 0 ? f : sum ? s + f : fmax(s, f);
         }
         s = warp_fold(s, sum);
-        if (lane == 0) t.sm->res[k] = s;
+        if (lane == 0) {
+            t.sm->res[k] = s;
+            fin(k, s);
+        }
     }
     __syncthreads();
     return true;
@@ -206,8 +228,8 @@ __device__ __forceinline__ double* team_partials(Team& t) {
 // folds that followed.  Up to kFlat values therefore go through shared
 // memory, where one warp per value sums MM_BLOCK / 32 of them per lane before
 // its only tree; more values share their trees (warp_sums_shared).
-template <int NS, int NX>
-__device__ bool team_reduce(Team& t, double (&s)[NS > 0 ? NS : 1], double (&x)[NX > 0 ? NX : 1]) {
+template <int NS, int NX, class Fin = NoFinish>
+__device__ bool team_reduce(Team& t, double (&s)[NS > 0 ? NS : 1], double (&x)[NX > 0 ? NX : 1], Fin fin = Fin()) {
     constexpr int K = NS + NX;
     static_assert(K <= MM_MAXRED, "too many reduction values");
     TeamSmem& sm = *t.sm;
@@ -252,7 +274,7 @@ __device__ bool team_reduce(Team& t, double (&s)[NS > 0 ? NS : 1], double (&x)[N
             if (lane == 0) part[(size_t)k * t.nb + t.rank] = f2;
         }
     }
-    if (!team_combine<K, NS>(t, part)) return false;
+    if (!team_combine<K, NS>(t, part, fin)) return false;
 #pragma unroll
     for (int k = 0; k < NS; ++k) s[k] = sm.res[k];
 #pragma unroll
@@ -262,8 +284,8 @@ __device__ bool team_reduce(Team& t, double (&s)[NS > 0 ? NS : 1], double (&x)[N
 
 // Team sums accumulated in FP32 per thread and warp (the FP32 phases, whose
 // sums are all of positive terms), in FP64 across warps and blocks.
-template <int NS>
-__device__ bool team_sum_f32(Team& t, float (&s)[NS], double (&out)[NS]) {
+template <int NS, class Fin>
+__device__ bool team_sum_f32(Team& t, float (&s)[NS], Fin fin) {
     TeamSmem& sm = *t.sm;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double* part = team_partials(t);
@@ -277,11 +299,43 @@ __device__ bool team_sum_f32(Team& t, float (&s)[NS], double (&out)[NS]) {
         const double f = warp_fold(lane < kWarps ? sm.w[warp][lane] : 0.0, true);
         if (lane == 0) part[(size_t)warp * t.nb + t.rank] = f;
     }
-    if (!team_combine<NS, NS>(t, part)) return false;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) out[k] = sm.res[k];
-    return true;
+    return team_combine<NS, NS>(t, part, fin);
 }
+
+// Team values of a CG step: d.q of the direction step gives the step length,
+// r.z of the update gives beta and takes the old value's place.
+__device__ __forceinline__ void cg_length(CgScalars& g, double dq) {
+    g.a = g.rz / dq;
+    g.af = (float)g.a;
+}
+__device__ __forceinline__ void cg_beta(CgScalars& g, double rz) {
+    g.beta = rz / g.rz;
+    g.betaf = (float)g.beta;
+    g.rz_old = g.rz;
+    g.rz = rz;
+}
+__device__ __forceinline__ bool is_zero(double v) { return (__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFll) == 0; }
+
+// What the team values of an FP32 solve's preconditioned residual are for: the
+// first (mode INIT_FIRST), one after a reliable update (INIT_NEXT), one of a CG
+// step (STEP).
+enum CgMode { CG_INIT_FIRST, CG_INIT_NEXT, CG_STEP };
+struct CgResidual {
+    CgScalars& g;
+    CgMode mode;
+    double upd2, tol2;
+    __device__ void operator()(int k, double s) const {
+        if (k == 0) {
+            if (mode == CG_INIT_FIRST) g.rz = s;
+            else cg_beta(g, s);
+        } else if (mode != CG_STEP) {
+            g.rmax = s;
+        } else {
+            g.stop = s < upd2 * g.rmax || s < tol2;
+            g.rmax = fmax(g.rmax, s);
+        }
+    }
+};
 
 struct Row {
     long long base;
@@ -328,9 +382,8 @@ __device__ __forceinline__ int team_item(const Team& t, const Share& h, int k) {
 // exceed the columns) and skip the FP64 multiply-add, which would occupy the
 // SM's FP64 pipe for 19 cycles to add zero.
 template <int CH, typename T, typename VT, typename XT>
-__device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const int* __restrict__ col,
-                                      const VT* __restrict__ val, const XT* x, int r, int pad) {
-    const Row A = sell_row(sptr, r);
+__device__ __forceinline__ T sell_dot_row(const Row& A, const int* __restrict__ col, const VT* __restrict__ val,
+                                          const XT* x, int pad) {
     T s = T(0);
     for (int k0 = 0; k0 < A.width; k0 += CH) {
         int c[CH];
@@ -353,9 +406,45 @@ __device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const 
 
 template <int CH, typename T, typename VT, typename XT>
 __device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const int* __restrict__ col,
+                                      const VT* __restrict__ val, const XT* x, int r, int pad) {
+    return sell_dot_row<CH, T>(sell_row(sptr, r), col, val, x, pad);
+}
+template <int CH, typename T, typename VT, typename XT>
+__device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const int* __restrict__ col,
                                       const VT* __restrict__ val, const XT* x, int r) {
     return sell_dot<CH, T>(sptr, col, val, x, r, r);
 }
+
+// f(p, s, v) for the team's potential rows p with s = (K_phi x)_p in FP64 and
+// v = pre(p), the row's vector operands.  A round is a chain of slice pointers,
+// entries and gathers, each an L2 round trip, then the FP64 pipe: the pointers
+// are read one round ahead and the vector operands before the product (left to
+// the compiler they came after it: 26.1 against 22.2 us for a direction step on
+// 250,047 rows of 15 entries).
+template <typename XT, class Pre, class F>
+__device__ __forceinline__ void phi_products(const Problem& P, const Team& t, const XT* x, Pre pre, F f) {
+    const Share h = t.sm->phi;
+    const int lane = threadIdx.x & 31;
+    auto item = [&](int k) { return k <= h.full ? team_item(t, h, k) : -1; };
+    auto slice = [&](int i) { return i < 0 ? Row{0, 0} : sell_row(P.p_sptr, 32 * i + lane); };
+    int i = item(0);
+    Row A = slice(i);
+    for (int k = 0; k <= h.full; ++k) {
+        const int ni = item(k + 1);
+        const Row N = slice(ni);
+        const int p = 32 * i + lane;
+        if (i >= 0 && p < P.nphi) {
+            const auto v = pre(p);
+            f(p, sell_dot_row<8, double>(A, P.p_col, P.Kp, x, p), v);
+        }
+        i = ni;
+        A = N;
+    }
+}
+struct NoOperands {};
+struct Operands {
+    double a, b, c;
+};
 
 // Same for a scalar matrix applied to a SoA 3-vector (stride n); T the
 // type of the sums and of the values (FP64, or FP32 in the precision form's
@@ -655,8 +744,8 @@ __device__ bool ph_pinit(Ctx& C, int s, double& bb, double& rz, double& rr) {
     const double* x = P.X[s];
     double acc[3] = {0.0, 0.0, 0.0};
     double dummy[1] = {0.0};
-    ROWS(p, t.sm->phi, P.nphi) {
-        const double kphi = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, P.phi, p);
+    auto pre = [](int) { return NoOperands{}; };
+    phi_products(P, t, P.phi, pre, [&](int p, double kphi, NoOperands) {
         double bp = 0.0;
         if (p < nm) {
             bp = row_div(P, x, p);
@@ -669,7 +758,7 @@ __device__ bool ph_pinit(Ctx& C, int s, double& bb, double& rz, double& rr) {
         acc[0] += bp * bp;
         acc[1] += r * z;
         acc[2] += r * r;
-    }
+    });
     if (!team_reduce<3, 0>(t, acc, dummy)) return false;
     bb = acc[0];
     rz = acc[1];
@@ -681,33 +770,32 @@ __device__ bool ph_pinit(Ctx& C, int s, double& bb, double& rz, double& rr) {
 __device__ bool ph_pmatvec(Ctx& C, const double* v, double* q) {
     const Problem& P = *C.P;
     Team& t = C.t;
-    ROWS(p, t.sm->phi, P.nphi) q[p] = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, v, p);
+    phi_products(P, t, v, [](int) { return NoOperands{}; }, [&](int p, double s, NoOperands) { q[p] = s; });
     return team_sync(t);
 }
 
 // CG direction step of Algorithm 1 with the product formed by recurrence:
 // w = K z, d = z + beta d, q = w + beta q (= K d), in place.  Sum: d . q.
-__device__ bool ph_pdirection(Ctx& C, const double* z, double beta, double* d, double* q, double& dq) {
+__device__ bool ph_pdirection(Ctx& C, const double* z, double beta, double* d, double* q) {
     const Problem& P = *C.P;
     Team& t = C.t;
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
-    const bool first = (beta == 0.0);
-    ROWS(p, t.sm->phi, P.nphi) {
-        const double s = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, z, p);
-        const double dn = first ? z[p] : z[p] + beta * d[p];
-        const double qn = first ? s : s + beta * q[p];
+    const bool first = is_zero(beta);
+    auto pre = [&](int p) { return first ? Operands{z[p], 0.0, 0.0} : Operands{z[p], d[p], q[p]}; };
+    phi_products(P, t, z, pre, [&](int p, double s, const Operands& v) {
+        const double dn = first ? v.a : v.a + beta * v.b;
+        const double qn = first ? s : s + beta * v.c;
         d[p] = dn;
         q[p] = qn;
         acc[0] += dn * qn;
-    }
-    if (!team_reduce<1, 0>(t, acc, dummy)) return false;
-    dq = acc[0];
-    return true;
+    });
+    CgScalars& g = t.sm->cg;
+    return team_reduce<1, 0>(t, acc, dummy, [&g](int, double s) { cg_length(g, s); });
 }
 
-// phi += a v; r -= a q; z = diag^-1 r.  Sums: r.z, |r|^2.
-__device__ bool ph_pupdate(Ctx& C, const double* v, double a, double& rz, double& rr) {
+// phi += a v; r -= a q; z = diag^-1 r.  Sums: r.z, |r|^2 (against tol2).
+__device__ bool ph_pupdate(Ctx& C, const double* v, double a, double tol2) {
     const Problem& P = *C.P;
     Team& t = C.t;
     double acc[2] = {0.0, 0.0};
@@ -721,10 +809,11 @@ __device__ bool ph_pupdate(Ctx& C, const double* v, double a, double& rz, double
         acc[0] += r * z;
         acc[1] += r * r;
     }
-    if (!team_reduce<2, 0>(t, acc, dummy)) return false;
-    rz = acc[0];
-    rr = acc[1];
-    return true;
+    CgScalars& g = t.sm->cg;
+    return team_reduce<2, 0>(t, acc, dummy, [&g, tol2](int k, double s) {
+        if (k == 0) cg_beta(g, s);
+        else g.stop = !(s >= tol2);
+    });
 }
 
 __device__ bool ph_pzero(Ctx& C) {
@@ -909,7 +998,7 @@ __device__ __noinline__ bool ph_amg_dense(Ctx& C) {
 
 // Up phase of level l: y = omega D^-1 (b + rpre) + U y_{l+1}.  At level 0,
 // y is the preconditioned residual z; sums r.z and |r|^2.
-__device__ __noinline__ bool ph_amg_up(Ctx& C, int l, double& rz, double& rr) {
+__device__ __noinline__ bool ph_amg_up(Ctx& C, int l, const CgResidual& fin) {
     const Problem& P = *C.P;
     Team& t = C.t;
     const Level& V = P.lev[l];
@@ -936,30 +1025,26 @@ __device__ __noinline__ bool ph_amg_up(Ctx& C, int l, double& rz, double& rr) {
         }
     }
     if (l > 0) return team_sync(t);
-    double out[2];
-    if (!team_sum_f32<2>(t, acc, out)) return false;
-    rz = out[0];
-    rr = out[1];
-    return true;
+    return team_sum_f32<2>(t, acc, fin);
 }
 
 // z = V-cycle(r) for r = pres32, whose smoothed iterate amg_x0 = omega
 // D^-1 r has been written (and a barrier passed) by the caller.  Sums r.z,
 // |r|^2.
-__device__ bool amg_vcycle(Ctx& C, double& rz, double& rr) {
+__device__ bool amg_vcycle(Ctx& C, const CgResidual& fin) {
     const Problem& P = *C.P;
     for (int l = 0; l < P.nlev; ++l)
         if (!ph_amg_down(C, l)) return false;
     if (!ph_amg_dense(C)) return false;
     for (int l = P.nlev - 1; l >= 0; --l)
-        if (!ph_amg_up(C, l, rz, rr)) return false;
+        if (!ph_amg_up(C, l, fin)) return false;
     return true;
 }
 
 __device__ __forceinline__ bool use_amg(const Problem& P) { return P.prm.amg != 0 && P.nlev > 0; }
 
 // r32 = r, z32 = M^-1 r32 (Jacobi or the V-cycle), delta = 0.  Sums: r.z, |r|^2.
-__device__ bool ph_p32_init(Ctx& C, double& rz, double& rr) {
+__device__ bool ph_p32_init(Ctx& C, const CgResidual& fin) {
     const Problem& P = *C.P;
     Team& t = C.t;
     if (use_amg(P)) {
@@ -970,10 +1055,9 @@ __device__ bool ph_p32_init(Ctx& C, double& rz, double& rr) {
             P.pdelta32[p] = 0.0f;
         }
         if (!team_sync(t)) return false;
-        return amg_vcycle(C, rz, rr);
+        return amg_vcycle(C, fin);
     }
     float acc[2] = {0.0f, 0.0f};
-    double out[2];
     ROWS(p, t.sm->phi, P.nphi) {
         const float r = (float)P.pres[p];
         const float z = r * P.dinvP32[p];
@@ -983,18 +1067,14 @@ __device__ bool ph_p32_init(Ctx& C, double& rz, double& rr) {
         acc[0] += r * z;
         acc[1] += r * r;
     }
-    if (!team_sum_f32<2>(t, acc, out)) return false;
-    rz = out[0];
-    rr = out[1];
-    return true;
+    return team_sum_f32<2>(t, acc, fin);
 }
 
 // FP32 direction step: d = z + beta d, q = K32 z + beta q.  Sum: d . q.
-__device__ bool ph_p32_direction(Ctx& C, float beta, double& dq) {
+__device__ bool ph_p32_direction(Ctx& C, float beta) {
     const Problem& P = *C.P;
     Team& t = C.t;
     float acc[1] = {0.0f};
-    double out[1];
     const bool first = (beta == 0.0f);
     const float* z = P.pprec32;
     // per row: the new direction z + beta d and beta q, loaded ahead of the product
@@ -1008,13 +1088,12 @@ __device__ bool ph_p32_direction(Ctx& C, float beta, double& dq) {
         acc[0] += v.x * qn;
     };
     level0_products(P, t, P.k_sptr, P.k_col, P.Kp32, P.k_tab, z, P.nphi, true, pre, row);
-    if (!team_sum_f32<1>(t, acc, out)) return false;
-    dq = out[0];
-    return true;
+    CgScalars& g = t.sm->cg;
+    return team_sum_f32<1>(t, acc, [&g](int, double s) { cg_length(g, s); });
 }
 
 // delta += a d; r -= a q; z = M^-1 r.  Sums: r.z, |r|^2.
-__device__ bool ph_p32_update(Ctx& C, float a, double& rz, double& rr) {
+__device__ bool ph_p32_update(Ctx& C, float a, const CgResidual& fin) {
     const Problem& P = *C.P;
     Team& t = C.t;
     // Streaming pass in float4 (four rows per load; the FP32 vectors are
@@ -1046,10 +1125,9 @@ __device__ bool ph_p32_update(Ctx& C, float a, double& rz, double& rr) {
             P.amg_x0[p] = om * P.dinvP32[p] * r;
         }
         if (!team_sync(t)) return false;
-        return amg_vcycle(C, rz, rr);
+        return amg_vcycle(C, fin);
     }
     float acc[2] = {0.0f, 0.0f};
-    double out[2];
     float4* __restrict__ z4 = reinterpret_cast<float4*>(P.pprec32);
     ROWS(i, t.sm->phi4, n4) {
         const float4 d = dir4[i], q = q4[i], r = res4[i], e = del4[i], w = dv4[i];
@@ -1071,10 +1149,7 @@ __device__ bool ph_p32_update(Ctx& C, float a, double& rz, double& rr) {
         acc[0] += r * z;
         acc[1] += r * r;
     }
-    if (!team_sum_f32<2>(t, acc, out)) return false;
-    rz = out[0];
-    rr = out[1];
-    return true;
+    return team_sum_f32<2>(t, acc, fin);
 }
 
 // FP64 refinement: phi += delta; r -= K delta (FP64 operator).  Sum: |r|^2.
@@ -1084,13 +1159,13 @@ __device__ bool ph_p64_refine(Ctx& C, double& rr) {
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
     const float* dl = P.pdelta32;
-    ROWS(p, t.sm->phi, P.nphi) {
-        const double s = sell_dot<8, double>(P.p_sptr, P.p_col, P.Kp, dl, p);
-        P.phi[p] += (double)dl[p];
-        const double r = P.pres[p] - s;
+    auto pre = [&](int p) { return Operands{(double)dl[p], P.phi[p], P.pres[p]}; };
+    phi_products(P, t, dl, pre, [&](int p, double s, const Operands& v) {
+        P.phi[p] = v.b + v.a;
+        const double r = v.c - s;
         P.pres[p] = r;
         acc[0] += r * r;
-    }
+    });
     if (!team_reduce<1, 0>(t, acc, dummy)) return false;
     rr = acc[0];
     return true;
@@ -1109,21 +1184,20 @@ __device__ bool solve_potential_mixed(Ctx& C, double bb, double rr) {
     const double tol2 = C.ptol * C.ptol * bb;
     const double upd2 = P.prm.inner_tol * P.prm.inner_tol;
     if (rr < tol2) return true;
-    double rz, r32;
-    if (!ph_p32_init(C, rz, r32)) return false;
-    double rmax = r32;
+    CgScalars& g = C.t.sm->cg;
+    if (!ph_p32_init(C, {g, CG_INIT_FIRST, upd2, tol2})) return false;
     float beta = 0.0f;
     long long k = 0;
     int updates = 0;
     while (k < P.prm.poisson_max_iter) {
-        double dq;
-        if (!ph_p32_direction(C, beta, dq)) return false;
-        const float a = (float)(rz / dq);
-        double rzn;
-        if (!ph_p32_update(C, a, rzn, r32)) return false;
+        if (!ph_p32_direction(C, beta)) return false;
+        if (!ph_p32_update(C, g.af, {g, CG_STEP, upd2, tol2})) return false;
         ++k;
-        if (r32 < upd2 * rmax || r32 < tol2) {
-            // reliable update
+        beta = g.betaf;
+        if (g.stop) {
+            // reliable update; beta is that of the true residual to the one
+            // before this step, so the scalar r.z goes back to it
+            const double rz = g.rz_old;
             if (!ph_p64_refine(C, rr)) return false;
             C.mr++;
             ++updates;
@@ -1131,13 +1205,10 @@ __device__ bool solve_potential_mixed(Ctx& C, double bb, double rr) {
                 C.mi += k + updates;
                 return true;
             }
-            if (!ph_p32_init(C, rzn, r32)) return false;
-            rmax = r32;
-        } else {
-            rmax = fmax(rmax, r32);
+            if (threadIdx.x == 0) g.rz = rz;
+            if (!ph_p32_init(C, {g, CG_INIT_NEXT, upd2, tol2})) return false;
+            beta = g.betaf;
         }
-        beta = (float)(rzn / rz);
-        rz = rzn;
     }
     // iteration cap: fold the pending correction into phi
     if (!ph_p64_refine(C, rr)) return false;
@@ -1154,16 +1225,16 @@ __device__ bool solve_potential(Ctx& C, int s) {
     if (bb == 0.0) return ph_pzero(C);
     if (P.prm.precision == 1) return solve_potential_mixed(C, bb, rr);
     const double tol2 = C.ptol * C.ptol * bb;
+    CgScalars& g = C.t.sm->cg;
+    if (threadIdx.x == 0) g.rz = rz;             // (thread 0 also folds r.z and d.q)
     double beta = 0.0;
     long long k = 0;
-    while (rr >= tol2 && k < P.prm.poisson_max_iter) {
-        double pq;
-        if (!ph_pdirection(C, P.pprec, beta, P.pdir[0], P.pq, pq)) return false;
-        const double a = rz / pq;
-        double rzn;
-        if (!ph_pupdate(C, P.pdir[0], a, rzn, rr)) return false;
-        beta = rzn / rz;
-        rz = rzn;
+    bool stop = !(rr >= tol2);
+    while (!stop && k < P.prm.poisson_max_iter) {
+        if (!ph_pdirection(C, P.pprec, beta, P.pdir[0], P.pq)) return false;
+        if (!ph_pupdate(C, P.pdir[0], g.a, tol2)) return false;
+        beta = g.beta;
+        stop = g.stop != 0;
         ++k;
     }
     C.mi += k;
@@ -1266,12 +1337,37 @@ __device__ bool evaluate(Ctx& C, int c, int s, bool trial, double a, int ref = 0
     return true;
 }
 
+// Team values of the preconditioner's solve: of a direction step (step length,
+// li2), of the initial residual (|b| and li3's limit) and of an update (beta,
+// li3).
+struct InnerLength {
+    CgScalars& g;
+    __device__ void operator()(int, double dHd) const {
+        cg_length(g, dHd);
+        g.stop = dHd <= 0.0;
+    }
+};
+struct InnerResidual {
+    CgScalars& g;
+    bool initial;
+    __device__ void operator()(int k, double s) const {
+        if (k == 0) {
+            if (initial) g.rz = s;
+            else cg_beta(g, s);
+        } else {
+            const double r = sqrt(s);
+            if (initial) g.eps = fmin(0.5, sqrt(r)) * r;
+            g.stop = r < g.eps;
+        }
+    }
+};
+
 // w = H(m) v (Eq. precond, magnetostatics dropped; last term only if
 // keep_last_term).  With d given, the inner CG direction step follows by
 // recurrence: d = ca v + beta d and hd = ca w + beta hd (= H d), in place,
-// sum d . hd.  Without d, w is written to hd (sum v . w).
+// sum d . hd (step length and li2's sign).  Without d, w is written to hd.
 __device__ bool ph_hess(Ctx& C, int s, const double* v, double ca, double beta, double* d,
-                        double* hd, double& dHd) {
+                        double* hd) {
     const Problem& P = *C.P;
     Team& t = C.t;
     const int nm = P.nm;
@@ -1279,7 +1375,7 @@ __device__ bool ph_hess(Ctx& C, int s, const double* v, double ca, double beta, 
     const double* lamv = P.LAM[s];
     const double* gr = P.GR[s];
     const bool keep = P.prm.keep_last_term != 0;
-    const bool first = (beta == 0.0);
+    const bool first = is_zero(beta);
     double acc[1] = {0.0};
     double dummy[1] = {0.0};
     ROWS(i, t.sm->nm, nm) {
@@ -1321,12 +1417,9 @@ __device__ bool ph_hess(Ctx& C, int s, const double* v, double ca, double beta, 
             hd[i] = w0;
             hd[nm + i] = w1;
             hd[2 * nm + i] = w2;
-            acc[0] += v0 * w0 + v1 * w1 + v2 * w2;
         }
     }
-    if (!team_reduce<1, 0>(t, acc, dummy)) return false;
-    dHd = acc[0];
-    return true;
+    return team_reduce<1, 0>(t, acc, dummy, InnerLength{t.sm->cg});
 }
 
 // One application of an operator of Eq. (energy) (the operator entry
@@ -1369,7 +1462,7 @@ __device__ bool precond_solve(Ctx& C, int s) {
         C.y_is_g = 1;
         return true;
     }
-    const double* g = P.GP[s];
+    const double* gp = P.GP[s];
     // residual gr = H*0 + b with b = -g; preconditioned yv; direction -yv
     double acc[2] = {0.0, 0.0};
     double dummy[1] = {0.0};
@@ -1377,7 +1470,7 @@ __device__ bool precond_solve(Ctx& C, int s) {
         const double di = P.dinvA[i];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double r = -g[c * nm + i];
+            const double r = -gp[c * nm + i];
             const double z = di * r;
             P.ires[c * nm + i] = r;
             P.iprec[c * nm + i] = z;
@@ -1386,21 +1479,18 @@ __device__ bool precond_solve(Ctx& C, int s) {
             acc[1] += r * r;
         }
     }
-    if (!team_reduce<2, 0>(t, acc, dummy)) return false;
-    double gy = acc[0];
-    const double ng = sqrt(acc[1]);
-    const double eps = fmin(0.5, sqrt(ng)) * ng;
+    CgScalars& g = t.sm->cg;
+    if (!team_reduce<2, 0>(t, acc, dummy, InnerResidual{g, true})) return false;
     C.y_is_g = 0;
-    if (ng < eps) return true;                  // y = 0 (only when g = 0 ... eps = 0)
+    if (g.stop) return true;                    // y = 0 (only when g = 0 ... eps = 0)
     double beta = 0.0;
     int steps = 0;
     while (steps < jmax) {
-        double dHd;
         // direction d = -yv + beta d and H d, by recurrence
-        if (!ph_hess(C, s, P.iprec, -1.0, beta, P.idir[0], P.ihd, dHd)) return false;
+        if (!ph_hess(C, s, P.iprec, -1.0, beta, P.idir[0], P.ihd)) return false;
         ++steps;
         C.li++;
-        if (dHd <= 0.0) {                       // li2
+        if (g.stop) {                           // li2
             C.li2++;
             if (steps == 1) {
                 C.y_is_g = 1;
@@ -1408,7 +1498,7 @@ __device__ bool precond_solve(Ctx& C, int s) {
             }
             return true;
         }
-        const double a = gy / dHd;
+        const double a = g.a;
         const double* dv = P.idir[0];
         double a2[2] = {0.0, 0.0};
         ROWS(i, t.sm->nm, nm) {
@@ -1425,10 +1515,9 @@ __device__ bool precond_solve(Ctx& C, int s) {
                 a2[1] += r * r;
             }
         }
-        if (!team_reduce<2, 0>(t, a2, dummy)) return false;
-        if (sqrt(a2[1]) < eps) return true;     // li3
-        beta = a2[0] / gy;
-        gy = a2[0];
+        if (!team_reduce<2, 0>(t, a2, dummy, InnerResidual{g, false})) return false;
+        if (g.stop) return true;                // li3
+        beta = g.beta;
     }
     return true;                                // li1
 }
@@ -1440,7 +1529,7 @@ __device__ bool precond_solve(Ctx& C, int s) {
 // FP32 products summed in FP64, the step length and beta stay FP64 scalars
 // and the solution y accumulates in FP64 (the search direction is built from
 // it).  The exits li1-li3 and their counters are those of precond_solve.
-__device__ bool ph_hess32(Ctx& C, int s, const float* v, float beta, float* d, float* hd, double& dHd) {
+__device__ bool ph_hess32(Ctx& C, int s, const float* v, float beta, float* d, float* hd) {
     const Problem& P = *C.P;
     Team& t = C.t;
     const int nm = P.nm;
@@ -1484,9 +1573,7 @@ __device__ bool ph_hess32(Ctx& C, int s, const float* v, float beta, float* d, f
             acc[0] += (double)(dn * hn);
         }
     }
-    if (!team_reduce<1, 0>(t, acc, dummy)) return false;
-    dHd = acc[0];
-    return true;
+    return team_reduce<1, 0>(t, acc, dummy, InnerLength{t.sm->cg});
 }
 
 __device__ bool precond_solve32(Ctx& C, int s) {
@@ -1498,14 +1585,14 @@ __device__ bool precond_solve32(Ctx& C, int s) {
         C.y_is_g = 1;
         return true;
     }
-    const double* g = P.GP[s];
+    const double* gp = P.GP[s];
     double acc[2] = {0.0, 0.0};
     double dummy[1] = {0.0};
     ROWS(i, t.sm->nm, nm) {
         const float di = P.dinvA32[i];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float r = (float)(-g[c * nm + i]);
+            const float r = (float)(-gp[c * nm + i]);
             const float z = di * r;
             P.ires32[c * nm + i] = r;
             P.iprec32[c * nm + i] = z;
@@ -1514,20 +1601,17 @@ __device__ bool precond_solve32(Ctx& C, int s) {
             acc[1] += (double)(r * r);
         }
     }
-    if (!team_reduce<2, 0>(t, acc, dummy)) return false;
-    double gy = acc[0];
-    const double ng = sqrt(acc[1]);
-    const double eps = fmin(0.5, sqrt(ng)) * ng;
+    CgScalars& g = t.sm->cg;
+    if (!team_reduce<2, 0>(t, acc, dummy, InnerResidual{g, true})) return false;
     C.y_is_g = 0;
-    if (ng < eps) return true;
-    double beta = 0.0;
+    if (g.stop) return true;
+    float beta = 0.0f;
     int steps = 0;
     while (steps < jmax) {
-        double dHd;
-        if (!ph_hess32(C, s, P.iprec32, (float)beta, P.idir32, P.ihd32, dHd)) return false;
+        if (!ph_hess32(C, s, P.iprec32, beta, P.idir32, P.ihd32)) return false;
         ++steps;
         C.li++;
-        if (dHd <= 0.0) {                       // li2
+        if (g.stop) {                           // li2
             C.li2++;
             if (steps == 1) {
                 C.y_is_g = 1;
@@ -1535,8 +1619,8 @@ __device__ bool precond_solve32(Ctx& C, int s) {
             }
             return true;
         }
-        const double a = gy / dHd;
-        const float af = (float)a;
+        const double a = g.a;
+        const float af = g.af;
         double a2[2] = {0.0, 0.0};
         ROWS(i, t.sm->nm, nm) {
             const float di = P.dinvA32[i];
@@ -1552,10 +1636,9 @@ __device__ bool precond_solve32(Ctx& C, int s) {
                 a2[1] += (double)(r * r);
             }
         }
-        if (!team_reduce<2, 0>(t, a2, dummy)) return false;
-        if (sqrt(a2[1]) < eps) return true;     // li3
-        beta = a2[0] / gy;
-        gy = a2[0];
+        if (!team_reduce<2, 0>(t, a2, dummy, InnerResidual{g, false})) return false;
+        if (g.stop) return true;                // li3
+        beta = g.betaf;
     }
     return true;                                // li1
 }
@@ -1827,8 +1910,7 @@ __device__ __forceinline__ void solver_body(const Problem& P, int nb, int rank) 
             break;
         case MODE_HESS: {
             // input v in idir[0], output in ihd
-            double vHv;
-            if (!ph_hess(C, cur, P.idir[0], 1.0, 0.0, nullptr, P.ihd, vHv)) status = ST_TIMEOUT;
+            if (!ph_hess(C, cur, P.idir[0], 1.0, 0.0, nullptr, P.ihd)) status = ST_TIMEOUT;
             break;
         }
         case MODE_KPHI: {
