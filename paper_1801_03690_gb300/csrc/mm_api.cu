@@ -847,14 +847,47 @@ int select_kernel(mm_ctx* ctx, int variant) {
 constexpr int kAutoLargePhi = 2000000;
 int auto_blocks_per_sm(int nphi) { return nphi > kAutoLargePhi ? 4 : 2; }
 
+// The choice for an evaluation or minimisation in plain FP64.  A potential
+// step takes whole rounds of one row per thread, and a round that only part of
+// the threads has rows for takes as long as a full one, so the rounds decide:
+// ceil(rows / (SMs x 256 v)) of them at v x 256 threads per SM, each 1 : 1.35 :
+// 1.7 long at v = 2 : 3 : 4 (from direction steps on 250,047 rows: 4 rounds in
+// 22.2, 3 in 22.9 and 2 in 18.8 us).  Field steps measured at v = 2 / 3 / 4, ms:
+// 59,319 rows (jittered cube) 9.2 / 10.3 / 11.1, 79,507 rows 13.1 / 11.1 / 11.8,
+// 125,000 rows 17.0 / 19.4 / 15.2, 166,375 rows 24.1 / 21.6 / 23.2; a graded
+// polycrystal of 85,184 rows 11.6 / 10.2 / 11.0, of 117,649 13.0 / 14.4 / 12.7.
+// For many rows v = 4 wins, as measured on the 8.7 M-unknown polycrystal.
+int fp64_blocks_per_sm(int nphi, int nsm) {
+    constexpr double kRound[3] = {1.0, 1.35, 1.7};
+    int best = 2;
+    double cost = 0.0;
+    for (int v = 2; v <= 4; ++v) {
+        const long long per = 256ll * v * nsm;
+        const double c = (double)((nphi + per - 1) / per) * kRound[v - 2];
+        if (v == 2 || c < cost) {
+            best = v;
+            cost = c;
+        }
+    }
+    return best;
+}
+
 int launch_solver(mm_ctx* ctx, int mode, const mm::Params& prm) {
     ctx->P.prm = prm;
     ctx->P.mode = mode;
     CK_CUDA(cudaMemsetAsync(ctx->P.bar, 0, 64 * sizeof(unsigned), ctx->stream));
     CK_CUDA(cudaMemsetAsync(ctx->P.err, 0, sizeof(int), ctx->stream));
     void* args[] = {(void*)&ctx->P};
+    const void* kernel = ctx->kernel;
+    int threads = ctx->threads;
+    const bool chosen = ctx->blocks_per_sm_req >= 2 && ctx->blocks_per_sm_req <= 4;     // by the caller
+    if (!chosen && prm.precision == 0 && (mode == mm::MODE_MINIMIZE || mode == mm::MODE_EVAL)) {
+        const int variant = fp64_blocks_per_sm(ctx->P.nphi, ctx->nsm);
+        kernel = mm::solver_kernel(variant);
+        threads = mm::solver_threads(variant);
+    }
     CK_CUDA(cudaEventRecord(ctx->ev0, ctx->stream));
-    CK_CUDA(cudaLaunchCooperativeKernel(ctx->kernel, dim3(ctx->blocks), dim3(ctx->threads), args, 0, ctx->stream));
+    CK_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(ctx->blocks), dim3(threads), args, 0, ctx->stream));
     CK_CUDA(cudaEventRecord(ctx->ev1, ctx->stream));
     CK_CUDA(cudaMemcpyAsync(ctx->h_state, ctx->d_state, sizeof(mm::DevState), cudaMemcpyDeviceToHost,
                             ctx->stream));
@@ -1465,6 +1498,8 @@ int mm_upload_mesh(mm_ctx* ctx, int64_t n_nodes, const double* xyz, int64_t n_te
     if ((rc = build_hierarchy(ctx, P, std::move(Kfull)))) return rc;
     if (ctx->blocks_per_sm_req < 2 || ctx->blocks_per_sm_req > 4) {
         if (select_kernel(ctx, auto_blocks_per_sm(nphi)) != MM_OK) return fail(ctx, MM_ERR_CUDA, "no solver grid");
+        cudaFuncAttributes fa;           // loads the FP64 form's kernel here rather than in its first launch
+        CK_CUDA(cudaFuncGetAttributes(&fa, mm::solver_kernel(fp64_blocks_per_sm(nphi, ctx->nsm))));
     }
     if ((rc = dalloc(ctx, &P.partials, 2 * (size_t)MM_MAXRED * ctx->blocks))) return rc;
     if ((rc = dalloc(ctx, &P.bar, 64))) return rc;

@@ -424,3 +424,24 @@ def test_jmax_autotune_restores_the_state(lib):
     assert np.abs(m_a - mag2.get_magnetization()).max() < 1e-6
     mag.close()
     mag2.close()
+
+
+@pytest.mark.parametrize("n_mag,n_phi", [(20, 39 ** 3), (22, 43 ** 3), (26, 51 ** 3)])
+def test_fp64_threads_per_sm_agree(n_mag, n_phi):
+    """Plain FP64 launches choose 512, 768 or 1024 threads per SM from the
+    rounds of rows they take (these sizes: one each on 152 SMs); the gradient is
+    that of 512 threads asked for.  Both solve the potential to 1e-12 of its
+    right-hand side in another order of the sums; on these lattices a residual
+    enters the potential amplified by the square root of the condition number,
+    below 100 for the Jacobi-scaled operator: bound 1e-9 of the largest."""
+    from paper_1801_03690_gb300 import Magnet, Params
+    wl = synth.small_cube(n_mag=n_mag, h=2.5e-9, seed=2)
+    grads = []
+    for bps in (0, 2):
+        mag = Magnet(device=0, blocks_per_sm=bps)
+        mag.upload_workload(wl)
+        assert mag.sizes()["n_phi"] == n_phi
+        mag.set_field(np.array([0.05, 0.0, 0.02]))
+        grads.append(mag.gradient(wl.m0, params=Params(poisson_tol=1e-12)))
+        mag.close()
+    assert np.abs(grads[0] - grads[1]).max() <= 1e-9 * np.abs(grads[1]).max()
