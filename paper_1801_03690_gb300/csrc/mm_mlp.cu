@@ -1257,6 +1257,7 @@ extern "C" {
 int mm_mlp_fit_input_norm(mm_mlp* M, const float* X_dev, int64_t n) {
     if (!M || !X_dev || n < 2) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
+    MK(cudaStreamSynchronize(cudaStreamLegacy));     // the data may still be in the making on the default stream
     MK(cudaStreamSynchronize(M->stream));
     int rc = launch_stats<NIN / 4, STAT_NORM>(M, X_dev, n);
     if (rc) return rc;
@@ -1294,6 +1295,7 @@ int mm_mlp_fit_target_scales(mm_mlp* M, const float* T_dev, int64_t n, float* Tn
                              double* scale_phi) {
     if (!M || !T_dev || !Tn_dev || !scale_m || !scale_phi || n < 2) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
+    MK(cudaStreamSynchronize(cudaStreamLegacy));     // the data may still be in the making on the default stream
     MK(cudaStreamSynchronize(M->stream));
     int rc = launch_stats<1, STAT_TARGETS>(M, T_dev, n);
     if (rc) return rc;
