@@ -433,7 +433,10 @@ int mm_mlp_forward(mm_mlp* mlp, const float* X_dev, int64_t n, float* Y_dev);
 int mm_mlp_gradient(mm_mlp* mlp, const float* X_dev, const float* T_dev, int64_t n,
                     float* grad_host, float* loss_out);
 /* One Adam step (beta 0.9 / 0.999) on the mean squared error; loss_out may
- * be NULL (then no synchronisation). */
+ * be NULL (then no synchronisation: the step reads its inputs after the work
+ * that the default stream has been given before the call, and work given to
+ * that stream afterwards runs after the step, so the inputs may be produced
+ * and overwritten there without waiting). */
 int mm_mlp_train_step(mm_mlp* mlp, const float* X_dev, const float* T_dev, int64_t n,
                       float lr, float* loss_out);
 /* Set the input standardisation from data: per feature, the mean and the

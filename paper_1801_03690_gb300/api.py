@@ -556,9 +556,19 @@ class MLP:
         return g, loss.value
 
     def train_step(self, X, T, lr, want_loss=False):
+        """One Adam step; without `want_loss` nothing waits for it, and it is
+        ordered after the current stream's work so far and before what that
+        stream is given next."""
+        import torch
         loss = C.c_float()
+        cur = torch.cuda.current_stream(X.device)
+        side = cur.cuda_stream != 0       # the library orders the step against the default stream
+        if side:
+            torch.cuda.default_stream(X.device).wait_stream(cur)
         rc = self._lib.mm_mlp_train_step(self._h, C.c_void_p(X.data_ptr()), C.c_void_p(T.data_ptr()),
                                          X.shape[0], C.c_float(lr), C.byref(loss) if want_loss else None)
+        if side:
+            cur.wait_stream(torch.cuda.default_stream(X.device))
         if rc:
             raise MMError(rc, "mm_mlp_train_step")
         return loss.value if want_loss else None

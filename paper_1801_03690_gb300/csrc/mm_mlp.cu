@@ -860,6 +860,7 @@ struct mm_mlp {
     float* tiles = nullptr;       // squared errors of every 128 rows
     float* loss = nullptr;        // the loss, and after it the error flag
     cudaStream_t stream = nullptr;
+    cudaEvent_t ev = nullptr;     // orders the stream against the caller's
     // inference buffers for the warm start
     long long fcap = 0;
     float *F = nullptr, *FY = nullptr;
@@ -883,6 +884,24 @@ namespace {
 size_t fwd_smem() { return sizeof(FwdSmem); }
 size_t bwd_smem() { return sizeof(BwdSmem); }
 size_t wgrad_smem() { return (size_t)2 * KCH * (128 + 8) * sizeof(__nv_bfloat16); }
+
+// The network's stream does not block on the default stream, so a pass that
+// neither side waits for is ordered by events: what the stream is given next
+// runs after the work that the default stream has been given so far (an event
+// there also stands behind the streams that block on it) ...
+int after_caller(mm_mlp* M) {
+    MK(cudaEventRecord(M->ev, cudaStreamLegacy));
+    MK(cudaStreamWaitEvent(M->stream, M->ev, 0));
+    return MM_OK;
+}
+
+// ... and what the default stream is given next runs after the stream's work,
+// so that the caller's buffers may be written or given back without a wait.
+int before_caller(mm_mlp* M) {
+    MK(cudaEventRecord(M->ev, M->stream));
+    MK(cudaStreamWaitEvent(cudaStreamLegacy, M->ev, 0));
+    return MM_OK;
+}
 
 // Blocks of a statistics pass: two resident per SM.
 int stat_blocks(const mm_mlp* M) { return 2 * M->nsm; }
@@ -1056,7 +1075,9 @@ int mm_mlp_create(mm_mlp** out, int device, uint64_t seed) {
         mm_mlp_destroy(M);
         return code;
     };
-    if (cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking) != cudaSuccess) return bail(MM_ERR_CUDA);
+    if (cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&M->ev, cudaEventDisableTiming) != cudaSuccess)
+        return bail(MM_ERR_CUDA);
     if (cudaMalloc(&M->p, NPARAM * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->wb, NPARAM * sizeof(__nv_bfloat16)) != cudaSuccess ||
         cudaMalloc(&M->g, NPARAM * sizeof(float)) != cudaSuccess ||
@@ -1116,6 +1137,7 @@ void mm_mlp_destroy(mm_mlp* M) {
                     (void*)M->DZ3, (void*)M->DZ4, (void*)M->Yb, (void*)M->part, (void*)M->F, (void*)M->FY,
                     (void*)M->d_prob, (void*)M->d_max, (void*)M->tpart, (void*)M->tiles, (void*)M->stats})
         if (q) cudaFree(q);
+    if (M->ev) cudaEventDestroy(M->ev);
     if (M->stream) cudaStreamDestroy(M->stream);
     delete M;
 }
@@ -1182,10 +1204,11 @@ int mm_mlp_train_step(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t
     const float b1 = 0.9f, b2 = 0.999f;
     const float step = (float)(M->step + 1);
     const Adam adam{M->p, M->am, M->av, M->wb, lr, b1, b2, 1e-8f, 1.0f - std::pow(b1, step), 1.0f - std::pow(b2, step)};
-    const int rc = gradient(M, X_dev, T_dev, n, &adam);
+    int rc = after_caller(M);
     if (rc) return rc;
+    if ((rc = gradient(M, X_dev, T_dev, n, &adam))) return rc;
     M->step++;
-    return loss_out ? read_loss(M, loss_out) : MM_OK;
+    return loss_out ? read_loss(M, loss_out) : before_caller(M);
 }
 
 }  // extern "C"

@@ -288,3 +288,35 @@ def test_statistics_edges(n, centre, scale):
     Xd[n - 1, 3] = float("nan")
     with pytest.raises(Exception):
         net.fit_input_norm(Xd)
+
+
+@pytest.mark.parametrize("side", [False, True])
+def test_train_step_is_ordered_against_the_caller(side):
+    """A step without a loss reads its batch after the work queued before the
+    call (a long one and the copies that fill the batch) and before what is
+    queued after it (the batch is overwritten at once), on the default stream
+    and on one that does not block on it.  The pass sums in a fixed order, so
+    the parameters are those of a run that waits at every point."""
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    g = torch.Generator(device="cuda").manual_seed(4)
+    data = [(torch.randn((3000, 16), generator=g, device="cuda"), torch.randn((3000, 4), generator=g, device="cuda"))
+            for _ in range(4)]
+    want = MLP(seed=8)
+    for X, T in data:
+        torch.cuda.synchronize()
+        want.train_step(X, T, 1e-3, want_loss=True)
+    net = MLP(seed=8)
+    Xb, Tb = torch.zeros((3000, 16), device="cuda"), torch.zeros((3000, 4), device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream() if side else torch.cuda.default_stream()):
+        for X, T in data:
+            torch.cuda._sleep(10_000_000)
+            Xb.copy_(X)
+            Tb.copy_(T)
+            net.train_step(Xb, Tb, 1e-3)
+            Xb.fill_(float("nan"))
+            Tb.fill_(float("nan"))
+        got = net.get_params()
+    torch.cuda.synchronize()
+    assert np.array_equal(got, want.get_params())
