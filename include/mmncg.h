@@ -419,9 +419,14 @@ int mm_mlp_set_params(mm_mlp* mlp, const float* params, int64_t count);
  * (default) = tcgen05 MMAs with FP32 accumulators in tensor memory (M = 128
  * per MMA), 1 = the warp-level mma.sync path, kept as a measured
  * comparison.  Both round at the same points (BF16 inputs, weights and
- * hidden activations; FP32 accumulation).  A tensor-core wait that runs out (2 s) makes the next
- * synchronising MLP call return MM_ERR_DEVICE_TIMEOUT. */
+ * hidden activations; FP32 accumulation). */
 int mm_mlp_set_tensor_path(mm_mlp* mlp, int path);
+/* Limit of a tensor-core wait in ns (default 2 s); 0: every wait counts as
+ * run out, which lets a caller test what it does then.  A wait that runs out
+ * makes the next forward pass, gradient, training step with a loss or
+ * mm_mlp_get_params return MM_ERR_DEVICE_TIMEOUT, once; the training steps
+ * from it up to that call leave weights, moments and step count as they were. */
+int mm_mlp_set_wait_limit(mm_mlp* mlp, int64_t ns);
 int mm_mlp_get_params(mm_mlp* mlp, float* params, int64_t count);
 /* Input standardisation applied in FP32 before the BF16 first layer:
  * x_c <- (x_c - mean[c]) / std[c] (default mean 0, std 1). */

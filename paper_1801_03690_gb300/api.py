@@ -482,6 +482,12 @@ class MLP:
         if rc:
             raise MMError(rc, "mm_mlp_set_tensor_path")
 
+    def set_wait_limit(self, ns):
+        """Limit of a tensor-core wait in ns (0: every wait counts as run out)."""
+        rc = self._lib.mm_mlp_set_wait_limit(self._h, int(ns))
+        if rc:
+            raise MMError(rc, "mm_mlp_set_wait_limit")
+
     def fit_input_norm(self, X):
         """Input standardisation from the data X [n, 16] (float32, device)."""
         assert X.is_cuda and X.is_contiguous() and X.shape[1] == 16

@@ -463,11 +463,14 @@ __global__ void __launch_bounds__(256) k_mlp_loss(long long n, const float* __re
     fold_loss(n, tiles, out);
 }
 
-// Adam on the FP32 master weights; refreshes the BF16 copies.
+// Adam on the FP32 master weights; refreshes the BF16 copies.  `step` is the
+// number of this step, kept in *steps once it is taken.
 struct Adam {
     float *p, *m, *v;
     __nv_bfloat16* wb;
     float lr, b1, b2, eps, c1, c2;
+    int* steps;
+    int step;
 };
 
 __device__ __forceinline__ void adam_update(const Adam& a, int i, float gi) {
@@ -480,8 +483,10 @@ __device__ __forceinline__ void adam_update(const Adam& a, int i, float gi) {
     a.wb[i] = __float2bfloat16(w);
 }
 
-__global__ void k_mlp_adam(int np, const float* g, const Adam a) {
+__global__ void k_mlp_adam(int np, const float* g, const int* err, const Adam a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (*err) return;                    // as in tc::k_mlp_reduce
+    if (i == 0) *a.steps = a.step;
     if (i < np) adam_update(a, i, g[i]);
 }
 
@@ -839,6 +844,13 @@ __global__ void k_scale_targets(long long n, const float* __restrict__ T, float 
     Tn[i * NOUT + 3] = T[i * NOUT + 3] / sp;
 }
 
+// What a pass leaves for the host.
+struct Result {
+    float loss;
+    int err;                      // set by a tensor-core wait that ran out
+    int steps;                    // Adam steps taken
+};
+
 struct mm_mlp {
     int device = 0;
     int nsm = 0;
@@ -858,7 +870,7 @@ struct mm_mlp {
     float* tpart = nullptr;       // tcgen05 training path: partial gradients, one set per CTA
     long long tcap = 0;
     float* tiles = nullptr;       // squared errors of every 128 rows
-    float* loss = nullptr;        // the loss, and after it the error flag
+    Result *res = nullptr, *h_res = nullptr;    // on the device, and the (pinned) copy of the last finish()
     cudaStream_t stream = nullptr;
     cudaEvent_t ev = nullptr;     // orders the stream against the caller's
     // inference buffers for the warm start
@@ -867,7 +879,8 @@ struct mm_mlp {
     mm::Problem* d_prob = nullptr;
     unsigned* d_max = nullptr;
     double* stats = nullptr;      // statistics: a result, the arrival counter, the blocks' partials
-    int* d_err = nullptr;         // set by a tensor-core wait that ran out (in loss[1])
+    bool unread = false;          // a pass that may set the error flag was launched after the last finish()
+    unsigned long long wait_ns = tc::kWaitNs;   // limit of such a wait
     int path = 0;                 // 0: tcgen05, 1: mma.sync (comparison)
 };
 
@@ -956,10 +969,12 @@ int ensure_tiles(mm_mlp* M, long long n) {
 
 int launch_forward(mm_mlp* M, const float* X, long long n, float* Y) {
     if (M->path == 0) {
+        M->unread = true;
         const int grid = (int)std::min((n + tc::TM - 1) / tc::TM, (long long)M->nsm);
         const int vec = (reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) % 16 == 0;
         tc::k_mlp_forward_tc<<<grid, tc::GROUPS * tc::TM, sizeof(tc::Smem), M->stream>>>(n, X, vec, M->wb, M->p,
-                                                                                       M->norm, Y, M->d_err);
+                                                                                       M->norm, Y, &M->res->err,
+                                                                                       M->wait_ns);
         MK(cudaGetLastError());
         return MM_OK;
     }
@@ -997,57 +1012,51 @@ int gradient_mma_sync(mm_mlp* M, const float* X, const float* T, long long n) {
         MK(cudaGetLastError());
     }
     k_mlp_tile_loss<<<(unsigned)((n + 127) / 128), 128, 0, M->stream>>>(n, M->Yb, T, M->tiles);
-    k_mlp_loss<<<1, 256, 0, M->stream>>>(n, M->tiles, M->loss);
+    k_mlp_loss<<<1, 256, 0, M->stream>>>(n, M->tiles, &M->res->loss);
     MK(cudaGetLastError());
     return MM_OK;
 }
 
-// Gradients into M->g and the loss into M->loss; adam != nullptr: the update
+// Gradients into M->g and the loss into M->res; adam != nullptr: the update
 // follows.
 int gradient(mm_mlp* M, const float* X, const float* T, long long n, const Adam* adam) {
     int rc;
     if ((rc = ensure_tiles(M, n))) return rc;
     if (M->path == 0) {
+        M->unread = true;
         const int grid = (int)std::min((n + tc::TM - 1) / tc::TM, (long long)M->nsm);
         const int vec = (reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(T)) % 16 == 0;
         tc::k_mlp_train_tc<<<grid, tc::TT, sizeof(tc::TrainSmem), M->stream>>>(n, X, T, vec, M->wb, M->p, M->norm,
-                                                                             M->tpart, M->tiles, M->d_err);
+                                                                             M->tpart, M->tiles, &M->res->err,
+                                                                             M->wait_ns);
         MK(cudaGetLastError());
-        tc::k_mlp_reduce<<<(NPARAM + 63) / 64 + 1, 256, 0, M->stream>>>(n, grid, M->tpart, M->tiles, M->g, M->loss,
-                                                                       adam != nullptr, adam ? *adam : Adam{});
+        tc::k_mlp_reduce<<<(NPARAM + 63) / 64 + 1, 256, 0, M->stream>>>(n, grid, M->tpart, M->tiles, M->g,
+                                                                       &M->res->loss, &M->res->err, adam != nullptr,
+                                                                       adam ? *adam : Adam{});
         MK(cudaGetLastError());
         return MM_OK;
     }
     if ((rc = gradient_mma_sync(M, X, T, n))) return rc;
     if (adam) {
-        k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, M->stream>>>(NPARAM, M->g, *adam);
+        k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, M->stream>>>(NPARAM, M->g, &M->res->err, *adam);
         MK(cudaGetLastError());
     }
     return MM_OK;
 }
 
-// MM_ERR_DEVICE_TIMEOUT if a tensor-core wait of the last launches ran out
-// (the flag is cleared); call after synchronising the stream.
-int check_err(mm_mlp* M) {
-    int e = 0;
-    MK(cudaMemcpy(&e, M->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-    if (!e) return MM_OK;
-    MK(cudaMemset(M->d_err, 0, sizeof(int)));
-    return MM_ERR_DEVICE_TIMEOUT;
-}
-
-// Wait for the stream; the last pass's loss, and check_err's status from the
-// same copy (the flag is the word after the loss).
-int read_loss(mm_mlp* M, float* loss) {
-    struct {
-        float loss;
-        int err;
-    } h;
-    MK(cudaMemcpyAsync(&h, M->loss, sizeof(h), cudaMemcpyDeviceToHost, M->stream));
+// Wait for the stream; *M->h_res is then the last pass's result.
+// MM_ERR_DEVICE_TIMEOUT if a tensor-core wait has run out since the last call
+// that said so (the flag is cleared): the Adam steps since then were not taken,
+// and the count goes back to those that were.
+int finish(mm_mlp* M) {
+    MK(cudaMemcpyAsync(M->h_res, M->res, sizeof(Result), cudaMemcpyDeviceToHost, M->stream));
     MK(cudaStreamSynchronize(M->stream));
-    if (h.err) return check_err(M);
-    *loss = h.loss;
-    return MM_OK;
+    M->unread = false;
+    if (!M->h_res->err) return MM_OK;
+    M->step = M->h_res->steps;
+    MK(cudaMemsetAsync(&M->res->err, 0, sizeof(int), M->stream));
+    MK(cudaStreamSynchronize(M->stream));
+    return MM_ERR_DEVICE_TIMEOUT;
 }
 
 }  // namespace
@@ -1061,6 +1070,12 @@ int mm_mlp_set_tensor_path(mm_mlp* M, int path) {
     MK(cudaSetDevice(M->device));
     MK(cudaStreamSynchronize(M->stream));
     M->path = path;
+    return MM_OK;
+}
+
+int mm_mlp_set_wait_limit(mm_mlp* M, int64_t ns) {
+    if (!M || ns < 0) return MM_ERR_ARG;
+    M->wait_ns = (unsigned long long)ns;
     return MM_OK;
 }
 
@@ -1083,15 +1098,15 @@ int mm_mlp_create(mm_mlp** out, int device, uint64_t seed) {
         cudaMalloc(&M->g, NPARAM * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->am, NPARAM * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->av, NPARAM * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&M->loss, 2 * sizeof(float)) != cudaSuccess ||
+        cudaMalloc(&M->res, sizeof(Result)) != cudaSuccess ||
+        cudaMallocHost(&M->h_res, sizeof(Result)) != cudaSuccess ||
         cudaMalloc(&M->d_prob, sizeof(mm::Problem)) != cudaSuccess ||
         cudaMalloc(&M->norm, 2 * NIN * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&M->d_max, sizeof(unsigned)) != cudaSuccess ||
         cudaMalloc(&M->stats, (ST_OUT + 1 + 32 * (size_t)stat_blocks(M)) * sizeof(double)) != cudaSuccess)
         return bail(MM_ERR_OOM);
     if (cudaMemset(M->stats, 0, (ST_OUT + 1) * sizeof(double)) != cudaSuccess) return bail(MM_ERR_CUDA);
-    M->d_err = reinterpret_cast<int*>(M->loss + 1);
-    if (cudaMemset(M->d_err, 0, sizeof(int)) != cudaSuccess) return bail(MM_ERR_CUDA);
+    if (cudaMemset(M->res, 0, sizeof(Result)) != cudaSuccess) return bail(MM_ERR_CUDA);
     {
         float id[2 * NIN];
         for (int i = 0; i < NIN; ++i) {
@@ -1132,11 +1147,12 @@ void mm_mlp_destroy(mm_mlp* M) {
     if (!M) return;
     cudaSetDevice(M->device);
     if (M->stream) cudaStreamSynchronize(M->stream);
-    for (void* q : {(void*)M->p, (void*)M->norm, (void*)M->wb, (void*)M->g, (void*)M->am, (void*)M->av, (void*)M->loss,
+    for (void* q : {(void*)M->p, (void*)M->norm, (void*)M->wb, (void*)M->g, (void*)M->am, (void*)M->av, (void*)M->res,
                     (void*)M->X0, (void*)M->A1, (void*)M->A2, (void*)M->A3, (void*)M->DZ1, (void*)M->DZ2,
                     (void*)M->DZ3, (void*)M->DZ4, (void*)M->Yb, (void*)M->part, (void*)M->F, (void*)M->FY,
                     (void*)M->d_prob, (void*)M->d_max, (void*)M->tpart, (void*)M->tiles, (void*)M->stats})
         if (q) cudaFree(q);
+    if (M->h_res) cudaFreeHost(M->h_res);
     if (M->ev) cudaEventDestroy(M->ev);
     if (M->stream) cudaStreamDestroy(M->stream);
     delete M;
@@ -1149,6 +1165,7 @@ int mm_mlp_set_params(mm_mlp* M, const float* params, int64_t count) {
     k_to_bf16<<<(NPARAM + 255) / 256, 256, 0, M->stream>>>(NPARAM, M->p, M->wb);
     MK(cudaMemsetAsync(M->am, 0, NPARAM * sizeof(float), M->stream));
     MK(cudaMemsetAsync(M->av, 0, NPARAM * sizeof(float), M->stream));
+    MK(cudaMemsetAsync(M->res, 0, sizeof(Result), M->stream));      // nothing of a failed pass is left
     MK(cudaStreamSynchronize(M->stream));
     M->step = 0;
     return MM_OK;
@@ -1171,6 +1188,8 @@ int mm_mlp_set_input_norm(mm_mlp* M, const float* mean, const float* stdev) {
 int mm_mlp_get_params(mm_mlp* M, float* params, int64_t count) {
     if (!M || !params || count != NPARAM) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
+    const int rc = M->unread ? finish(M) : MM_OK;
+    if (rc) return rc;
     MK(cudaStreamSynchronize(M->stream));
     MK(cudaMemcpy(params, M->p, NPARAM * sizeof(float), cudaMemcpyDeviceToHost));
     return MM_OK;
@@ -1179,10 +1198,8 @@ int mm_mlp_get_params(mm_mlp* M, float* params, int64_t count) {
 int mm_mlp_forward(mm_mlp* M, const float* X_dev, int64_t n, float* Y_dev) {
     if (!M || !X_dev || !Y_dev || n < 1) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    int rc = launch_forward(M, X_dev, n, Y_dev);
-    if (rc) return rc;
-    MK(cudaStreamSynchronize(M->stream));
-    return check_err(M);
+    const int rc = launch_forward(M, X_dev, n, Y_dev);
+    return rc ? rc : finish(M);
 }
 
 int mm_mlp_gradient(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t n, float* grad_host,
@@ -1191,10 +1208,9 @@ int mm_mlp_gradient(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t n
     MK(cudaSetDevice(M->device));
     int rc = gradient(M, X_dev, T_dev, n, nullptr);
     if (rc) return rc;
-    float loss = 0.0f;
-    if ((rc = read_loss(M, &loss))) return rc;
+    if ((rc = finish(M))) return rc;
     if (grad_host) MK(cudaMemcpy(grad_host, M->g, NPARAM * sizeof(float), cudaMemcpyDeviceToHost));
-    if (loss_out) *loss_out = loss;
+    if (loss_out) *loss_out = M->h_res->loss;
     return MM_OK;
 }
 
@@ -1203,12 +1219,16 @@ int mm_mlp_train_step(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t
     MK(cudaSetDevice(M->device));
     const float b1 = 0.9f, b2 = 0.999f;
     const float step = (float)(M->step + 1);
-    const Adam adam{M->p, M->am, M->av, M->wb, lr, b1, b2, 1e-8f, 1.0f - std::pow(b1, step), 1.0f - std::pow(b2, step)};
+    const Adam adam{M->p, M->am, M->av, M->wb, lr, b1, b2, 1e-8f, 1.0f - std::pow(b1, step), 1.0f - std::pow(b2, step),
+                    &M->res->steps, (int)(M->step + 1)};
     int rc = after_caller(M);
     if (rc) return rc;
     if ((rc = gradient(M, X_dev, T_dev, n, &adam))) return rc;
     M->step++;
-    return loss_out ? read_loss(M, loss_out) : before_caller(M);
+    if (!loss_out) return before_caller(M);
+    if ((rc = finish(M))) return rc;
+    *loss_out = M->h_res->loss;
+    return MM_OK;
 }
 
 }  // extern "C"
@@ -1408,8 +1428,7 @@ int mm_warmstart_apply(mm_ctx* ctx, mm_mlp* M, const double mu0h_next[3], double
     int rc = mm_warmstart_features(ctx, mu0h_next, M->F);
     if (rc) return rc;
     if ((rc = launch_forward(M, M->F, v.nm, M->FY))) return rc;
-    MK(cudaStreamSynchronize(M->stream));
-    if ((rc = check_err(M))) return mm::ctx_fail(ctx, rc, "a tensor-core wait of the network ran out");
+    if ((rc = finish(M))) return mm::ctx_fail(ctx, rc, "a tensor-core wait of the network ran out");
     mm::DevState hs;
     MK(cudaMemcpy(&hs, v.d_state, sizeof(mm::DevState), cudaMemcpyDeviceToHost));
     const double s = 1.0 / (4e-7 * 3.14159265358979323846 * v.Mref);

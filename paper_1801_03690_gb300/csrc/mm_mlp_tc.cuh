@@ -33,7 +33,7 @@ namespace tc {
 constexpr int TM = 128;      // rows per tile = the MMA's M = TMEM lanes
 constexpr int N4 = 16;       // the last layer's N, padded
 constexpr int TCOLS = 128;   // TMEM columns allocated (one N = 128 accumulator)
-constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s per MMA wait
+constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s per MMA wait (mm_mlp_set_wait_limit)
 
 constexpr int GROUPS = 4;    // forward pass: tiles in flight per SM, 128 threads each
 
@@ -94,8 +94,10 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 
 // Wait for the completion of the mbarrier phase with the given parity;
-// false if it did not complete within kWaitNs.
-__device__ __forceinline__ bool wait_phase(unsigned long long* bar, unsigned parity) {
+// false if it did not complete within `limit` ns (limit 0: without a look).
+__device__ __forceinline__ bool wait_phase(unsigned long long* bar, unsigned parity,
+                                           unsigned long long limit = kWaitNs) {
+    if (limit == 0) return false;
     const unsigned a = smem_u32(bar);
     const unsigned long long t0 = now_ns();
     while (true) {
@@ -107,7 +109,7 @@ __device__ __forceinline__ bool wait_phase(unsigned long long* bar, unsigned par
             : "r"(a), "r"(parity)
             : "memory");
         if (ok) return true;
-        if (now_ns() - t0 > kWaitNs) return false;
+        if (now_ns() - t0 > limit) return false;
     }
 }
 
@@ -220,7 +222,8 @@ __global__ void __launch_bounds__(GROUPS * TM, 1) k_mlp_forward_tc(long long n, 
                                                                    const __nv_bfloat16* __restrict__ wb,
                                                                    const float* __restrict__ p,
                                                                    const float* __restrict__ norm,
-                                                                   float* __restrict__ Y, int* err) {
+                                                                   float* __restrict__ Y, int* err,
+                                                                   unsigned long long limit) {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     Smem& s = *reinterpret_cast<Smem*>(tc_smem);
     constexpr int NT = GROUPS * TM;
@@ -289,7 +292,7 @@ __global__ void __launch_bounds__(GROUPS * TM, 1) k_mlp_forward_tc(long long n, 
     };
     // ... and their completion (the whole group agrees).
     auto done = [&]() -> bool {
-        const bool all = group_and(g, wait_phase(&s.bar[g], parity));
+        const bool all = group_and(g, wait_phase(&s.bar[g], parity, limit));
         if (all) parity ^= 1u;
         after_sync();
         return all;
@@ -395,7 +398,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(long long n, const float
                                                          const __nv_bfloat16* __restrict__ wb,
                                                          const float* __restrict__ p, const float* __restrict__ norm,
                                                          float* __restrict__ partial, float* __restrict__ tiles,
-                                                         int* err) {
+                                                         int* err, unsigned long long limit) {
     extern __shared__ __align__(1024) unsigned char tc_tsmem[];
     TrainSmem& s = *reinterpret_cast<TrainSmem*>(tc_tsmem);
     const int tid = threadIdx.x, warp = tid >> 5, row = tid & (TM - 1), half = tid / TM;
@@ -452,7 +455,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(long long n, const float
             issue();
             commit(&s.bar);
         }
-        const bool mine = wait_phase(&s.bar, parity);
+        const bool mine = wait_phase(&s.bar, parity, limit);
         const bool all = __syncthreads_and(mine) != 0;
         if (all) parity ^= 1u;
         after_sync();
@@ -646,14 +649,19 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(long long n, const float
 }
 
 // Gradients from the CTAs' partials in a fixed order, with the Adam update if
-// `update`; the last block folds the loss.  64 parameters per block, four
+// `update`; the last block folds the loss.  No gradient or weight is written once a wait of
+// this or an earlier pass has run out: a CTA that gave up left its partials
+// incomplete (its loss is not read either).  64 parameters per block, four
 // threads per parameter (each a quarter of the partials, eight loads in
 // flight): one thread per parameter over 128 partials leaves a thread with 16
 // dependent rounds of loads.
 __global__ void __launch_bounds__(256) k_mlp_reduce(long long n, int nparts, const float* __restrict__ partial,
                                                     const float* __restrict__ tiles, float* __restrict__ g,
-                                                    float* __restrict__ loss, int update, const Adam a) {
+                                                    float* __restrict__ loss, const int* err, int update,
+                                                    const Adam a) {
+    const int failed = *err;
     if (blockIdx.x == gridDim.x - 1) {
+        if (update && !failed && threadIdx.x == 0) *a.steps = a.step;
         fold_loss(n, tiles, loss);
         return;
     }
@@ -670,7 +678,7 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(long long n, int nparts, con
     }
     sh[q][lane] = s;
     __syncthreads();
-    if (q != 0 || e >= NPARAM) return;
+    if (q != 0 || e >= NPARAM || failed) return;
     s = (sh[0][lane] + sh[1][lane]) + (sh[2][lane] + sh[3][lane]);
     // dW1, dW2 and dW3 come transposed ([in][out])
     int i = e;

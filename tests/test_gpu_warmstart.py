@@ -320,3 +320,37 @@ def test_train_step_is_ordered_against_the_caller(side):
         got = net.get_params()
     torch.cuda.synchronize()
     assert np.array_equal(got, want.get_params())
+
+
+def test_a_wait_that_runs_out_leaves_the_network_as_it_was():
+    """With a limit of 0 every tensor-core wait counts as run out (the kernel
+    still lets its products finish).  The call that reports it is the next one
+    that waits; the steps up to then change neither weights nor moments nor the
+    step count, so training goes on as if they had not been asked for."""
+    import torch
+    from paper_1801_03690_gb300 import MLP, MMError
+    g = torch.Generator(device="cuda").manual_seed(9)
+    X, T = torch.randn((700, 16), generator=g, device="cuda"), torch.randn((700, 4), generator=g, device="cuda")
+    net, twin = MLP(seed=8), MLP(seed=8)
+    for n in (net, twin):
+        n.train_step(X, T, 1e-2)
+        n.train_step(X, T, 1e-2)
+    before = net.get_params()
+    net.set_wait_limit(0)
+    net.train_step(X, T, 1e-2)
+    net.set_wait_limit(2_000_000_000)
+    net.train_step(X, T, 1e-2)                               # sound, but after one that was not and is not reported yet
+    with pytest.raises(MMError):
+        net.get_params()
+    assert np.array_equal(net.get_params(), before)
+    net.set_wait_limit(0)
+    for call in (lambda: net.train_step(X, T, 1e-2, want_loss=True), lambda: net.gradient(X, T), lambda: net.forward(X)):
+        with pytest.raises(MMError):
+            call()
+        assert np.array_equal(net.get_params(), before)      # reported once
+    net.set_wait_limit(2_000_000_000)
+    for _ in range(2):
+        assert net.train_step(X, T, 1e-2, want_loss=True) == twin.train_step(X, T, 1e-2, want_loss=True)
+    assert np.array_equal(net.get_params(), twin.get_params())
+    with pytest.raises(MMError):
+        net.set_wait_limit(-1)
