@@ -438,6 +438,18 @@ class Batch:
         return ms.value
 
 
+def _default_stream_waits(device):
+    """The library orders a call that does not wait for the device against the
+    default stream.  If another stream is current, let the default stream wait
+    for it and return it, else None."""
+    import torch
+    cur = torch.cuda.current_stream(device)
+    if cur.cuda_stream == 0:
+        return None
+    torch.cuda.default_stream(device).wait_stream(cur)
+    return cur
+
+
 class MLP:
     """The warm-start network (16 -> 128 -> 128 -> 128 -> 4), trained and
     evaluated by the library's tensor-core kernels."""
@@ -491,6 +503,7 @@ class MLP:
     def fit_input_norm(self, X):
         """Input standardisation from the data X [n, 16] (float32, device)."""
         assert X.is_cuda and X.is_contiguous() and X.shape[1] == 16
+        _default_stream_waits(X.device)
         rc = self._lib.mm_mlp_fit_input_norm(self._h, C.c_void_p(X.data_ptr()), X.shape[0])
         if rc:
             raise MMError(rc, "mm_mlp_fit_input_norm")
@@ -512,6 +525,7 @@ class MLP:
         Tn = torch.empty_like(T)
         sm = C.c_double()
         sp = C.c_double()
+        _default_stream_waits(T.device)
         rc = self._lib.mm_mlp_fit_target_scales(self._h, C.c_void_p(T.data_ptr()), T.shape[0],
                                                 C.c_void_p(Tn.data_ptr()), C.byref(sm), C.byref(sp))
         if rc:
@@ -567,14 +581,11 @@ class MLP:
         stream is given next."""
         import torch
         loss = C.c_float()
-        cur = torch.cuda.current_stream(X.device)
-        side = cur.cuda_stream != 0       # the library orders the step against the default stream
-        if side:
-            torch.cuda.default_stream(X.device).wait_stream(cur)
+        side = _default_stream_waits(X.device)
         rc = self._lib.mm_mlp_train_step(self._h, C.c_void_p(X.data_ptr()), C.c_void_p(T.data_ptr()),
                                          X.shape[0], C.c_float(lr), C.byref(loss) if want_loss else None)
-        if side:
-            cur.wait_stream(torch.cuda.default_stream(X.device))
+        if side is not None:
+            side.wait_stream(torch.cuda.default_stream(X.device))
         if rc:
             raise MMError(rc, "mm_mlp_train_step")
         return loss.value if want_loss else None

@@ -1300,10 +1300,9 @@ extern "C" {
 int mm_mlp_fit_input_norm(mm_mlp* M, const float* X_dev, int64_t n) {
     if (!M || !X_dev || n < 2) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    MK(cudaStreamSynchronize(cudaStreamLegacy));     // the data may still be in the making on the default stream
-    MK(cudaStreamSynchronize(M->stream));
-    int rc = launch_stats<NIN / 4, STAT_NORM>(M, X_dev, n);
+    int rc = after_caller(M);
     if (rc) return rc;
+    if ((rc = launch_stats<NIN / 4, STAT_NORM>(M, X_dev, n))) return rc;
     double flag;
     MK(cudaMemcpyAsync(&flag, M->stats + 32, sizeof(flag), cudaMemcpyDeviceToHost, M->stream));
     MK(cudaStreamSynchronize(M->stream));
@@ -1338,10 +1337,9 @@ int mm_mlp_fit_target_scales(mm_mlp* M, const float* T_dev, int64_t n, float* Tn
                              double* scale_phi) {
     if (!M || !T_dev || !Tn_dev || !scale_m || !scale_phi || n < 2) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    MK(cudaStreamSynchronize(cudaStreamLegacy));     // the data may still be in the making on the default stream
-    MK(cudaStreamSynchronize(M->stream));
-    int rc = launch_stats<1, STAT_TARGETS>(M, T_dev, n);
+    int rc = after_caller(M);
     if (rc) return rc;
+    if ((rc = launch_stats<1, STAT_TARGETS>(M, T_dev, n))) return rc;
     const int vec = (reinterpret_cast<uintptr_t>(T_dev) | reinterpret_cast<uintptr_t>(Tn_dev)) % 16 == 0;
     k_scale_by<<<(unsigned)((n + 255) / 256), 256, 0, M->stream>>>(n, T_dev, vec, M->stats, Tn_dev);
     MK(cudaGetLastError());

@@ -354,3 +354,51 @@ def test_a_wait_that_runs_out_leaves_the_network_as_it_was():
     assert np.array_equal(net.get_params(), twin.get_params())
     with pytest.raises(MMError):
         net.set_wait_limit(-1)
+
+
+@pytest.mark.parametrize("kind", ["default", "blocking", "side"])
+def test_statistics_wait_for_the_data(kind):
+    """The statistics of data that are still in the making on the default
+    stream, on one that blocks on it and on a current stream that does not:
+    the same as those of finished data (the sums have a fixed order)."""
+    import ctypes
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    g = torch.Generator(device="cuda").manual_seed(2)
+    X0, T0 = torch.randn((5000, 16), generator=g, device="cuda"), torch.randn((5000, 4), generator=g, device="cuda")
+    torch.cuda.synchronize()
+    net = MLP(seed=1)
+    net.fit_input_norm(X0)
+    want = (*net.input_norm(), *net.fit_target_scales(T0)[1:])
+    handle = ctypes.c_void_p()
+    if kind == "blocking":
+        assert int(torch.cuda.cudart().cudaStreamCreate(ctypes.addressof(handle))) == 0
+    stream = {"default": torch.cuda.default_stream, "side": torch.cuda.Stream,
+              "blocking": lambda: torch.cuda.ExternalStream(handle.value)}[kind]()
+    X, T = torch.zeros_like(X0), torch.zeros_like(T0)
+    torch.cuda.synchronize()
+
+    def make():
+        torch.cuda._sleep(10_000_000)
+        X.copy_(X0)
+        T.copy_(T0)
+
+    with torch.cuda.stream(stream):
+        make()
+        if kind == "side":
+            net.fit_input_norm(X)
+    if kind != "side":
+        net.fit_input_norm(X)
+    mean, istd = net.input_norm()
+    X.zero_(), T.zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        make()
+        if kind == "side":
+            got = net.fit_target_scales(T)
+    if kind != "side":
+        got = net.fit_target_scales(T)
+    assert np.array_equal(mean, want[0]) and np.array_equal(istd, want[1]) and got[1:] == want[2:]
+    torch.cuda.synchronize()
+    if kind == "blocking":
+        assert int(torch.cuda.cudart().cudaStreamDestroy(handle.value)) == 0
