@@ -228,7 +228,8 @@ int mm_amg_host_apply(int64_t n, const int64_t* row_ptr, const int32_t* col, con
  * at once in the level-0 products with K_phi and the smoothed prolongation,
  * two keeping twice the loads in flight; restrict_lanes 4, 8 or 16 (0 =
  * default 8) -- lanes that share one row of a restriction P^T (levels whose
- * rows average over 160 entries always take 32).  Kept by the context across
+ * rows average over 160 entries, or that have no more rows than the launch has
+ * warps for the problem, always take 32).  Kept by the context across
  * mm_upload_mesh; takes effect at the next solver launch.  MM_ERR_ARG for
  * other values. */
 int mm_set_tiles(mm_ctx* ctx, int32_t rows_per_thread, int32_t restrict_lanes);

@@ -933,12 +933,15 @@ __device__ __forceinline__ void amg_restrict_g(const Problem& P, const Team& t, 
 
 // Lanes per restriction row.  Levels with long rows (the coarse end of the
 // hierarchy: hundreds of entries) or with no more rows than the team has
-// warps take a whole warp per row, the others P.restrict_lanes lanes, 8 by
-// default (measured on the 8.7 M-unknown polycrystal: 8 lanes 190 us, 4 lanes
-// 211, 16 lanes 225 for the level-0 down phase).
+// warps take a whole warp per row, whatever P.restrict_lanes says: with 8 lanes
+// three quarters of the warps had no rows on the latter (field steps: 12
+// platelets 37.9 ms, 36.9 now; 3.2 M-unknown polycrystal 97.0, 96.6 now).  The
+// others take P.restrict_lanes lanes, 8 by default (measured on the
+// 8.7 M-unknown polycrystal: 8 lanes 190 us, 4 lanes 211, 16 lanes 225 for the
+// level-0 down phase).
 __device__ __forceinline__ int restrict_group(const Problem& P, const Team& t, int l) {
     const Level& V = P.lev[l];
-    if (V.wide || (P.restrict_lanes == 0 && V.nc <= t.nb * kWarps)) return 32;
+    if (V.wide || V.nc <= t.nb * kWarps) return 32;
     return P.restrict_lanes == 4 || P.restrict_lanes == 16 ? P.restrict_lanes : 8;
 }
 

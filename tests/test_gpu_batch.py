@@ -147,3 +147,25 @@ def test_batch_multigrid_form_matches_single_problem_runs():
         assert s2["F"] == pytest.approx(s1["F"], rel=1e-8)
         assert np.abs(mag.get_magnetization() - m1).max() < 1e-5
     batch.close()
+
+
+def test_reported_config_is_the_one_that_runs():
+    """get_config answers with the defaults resolved: setting what it answers
+    leaves a batch's results as they were, bit by bit."""
+    from paper_1801_03690_gb300 import Batch, Params
+    wls = [synth.platelet("ellipse", 80e-9, 40e-9, thickness=5e-9, h=2.5e-9),
+           synth.platelet("disc", 50e-9, 50e-9, thickness=5e-9, h=2.5e-9)]
+    prm = Params(precision=1, amg=1, poisson_tol=1e-12, inner_tol=1e-3, max_iter=3)
+    out = []
+    for explicit in (False, True):
+        mags = _magnets(wls)
+        assert all(mag.amg_levels() for mag in mags)
+        batch = Batch(mags)
+        if explicit:
+            c = batch.get_config()
+            batch.config(c["blocks_per_sm"], c["gamma"])
+            batch.set_tiles(c["rows_per_thread"], c["restrict_lanes"])
+        batch.minimize(prm)
+        out.append([mag.get_magnetization() for mag in mags])
+        batch.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
