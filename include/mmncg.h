@@ -446,8 +446,8 @@ int mm_mlp_gradient(mm_mlp* mlp, const float* X_dev, const float* T_dev, int64_t
 int mm_mlp_train_step(mm_mlp* mlp, const float* X_dev, const float* T_dev, int64_t n,
                       float lr, float* loss_out);
 /* Set the input standardisation from data: per feature, the mean and the
- * unbiased standard deviation of X_dev [n][16] (device, FP64 sums, blocks
- * in a fixed order); a feature whose deviation is below 1e-6 (|mean| + 1)
+ * unbiased standard deviation of X_dev [n][16] (device; sums of FP64
+ * precision or better, blocks in a fixed order); a feature whose deviation is below 1e-6 (|mean| + 1)
  * is only centred.  Waits for the work that the default stream, and the
  * streams that block on it, have been given.  n >= 2.  mm_mlp_get_input_norm reads back the mean and
  * 1/std in use. */

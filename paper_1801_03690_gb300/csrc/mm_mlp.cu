@@ -618,22 +618,40 @@ __global__ void k_ws_targets(long long n, const float* __restrict__ X0, const fl
 // of x - s and (x - s)^2 about a shift s near the mean (that of 16 rows spread
 // over the data).  Two FP64 passes with one column per sweep read every line
 // 16 times, and at one FP64 instruction per warp every 19 cycles the six of an
-// element cost more than its bytes.  Here x - s, its square and the running
-// sums are exact or compensated pairs of FP32 words (two-sum, two-product;
-// Ogita, Rump and Oishi 2005), folded into FP64 every 32 rows: 24 FP32
-// operations an element, which the loads cover.  Standardising and scaling a
-// training set took 952 us at 1,200,003 rows and 249 at 1,000 (work space
-// allocated per call included), now 169 and 101.  A result that is not finite
-// (the FP32 squares overflow above 1e19) or whose shift lies too far from the
-// mean goes to the plain FP64 passes below.
-struct Pair {
-    float h, l;
+// element cost more than its bytes.  Here x - s and its square are exact and
+// the running sums are kept in three FP32 words (two-sum, two-product; Ogita,
+// Rump and Oishi 2005), folded into FP64 every 32 rows: a fold loses at most
+// 2^-53 of the sum of magnitudes, where 32 FP64 additions may lose 32 times
+// that.  It takes 60 FP32 operations an element.  (Two words take 24 but hold
+// about 43 bits: equal squares in 4,980,736 rows gave a deviation off by 9e-14.)
+// Standardising and scaling a training set of 1,200,003 rows takes 196 us with
+// two blocks resident per SM (64 registers, 112 B spilled outside the row loop;
+// 209 with one), 802 with the FP64 passes and their work space per call.  The
+// target scales come out within 2.3 x 2^-53 of 64-bit ones at 1,000 to 3,000,000
+// rows (FP64 passes: within 7.9 x 2^-53).
+// A result that is not finite (the FP32 squares overflow above 1e19) goes to
+// the plain FP64 passes below, and so does one whose shift lies more than two
+// deviations off the mean, where subtracting its square would cost more than
+// 2.3 bits.  Squares below FP32's normal range lose at most 2^-149 a term, which
+// is nothing against a deviation within the callers' limits (1e-12, and 1e-6 of
+// the mean).
+__device__ __forceinline__ float two_sum(float x, float y, float& err) {
+    const float s = __fadd_rn(x, y), z = __fsub_rn(s, x);
+    err = __fadd_rn(__fsub_rn(x, __fsub_rn(s, z)), __fsub_rn(y, z));
+    return s;
+}
+struct Triple {
+    float h, m, l;
 };
-__device__ __forceinline__ void pair_add(Pair& a, float h, float l) {
-    const float x = __fadd_rn(a.h, h), z = __fsub_rn(x, a.h);
-    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(x, z)), __fsub_rn(h, z));
-    a.h = x;
-    a.l = __fadd_rn(a.l, __fadd_rn(e, l));
+__device__ __forceinline__ void add_low(Triple& a, float v) {
+    float e;
+    a.m = two_sum(a.m, v, e);
+    a.l = __fadd_rn(a.l, e);
+}
+__device__ __forceinline__ void add(Triple& a, float v) {
+    float e;
+    a.h = two_sum(a.h, v, e);
+    add_low(a, e);
 }
 
 constexpr int ST = 512;              // threads per block
@@ -647,7 +665,7 @@ enum StatUse { STAT_NORM, STAT_TARGETS };
 // goes to norm; for STAT_TARGETS out[0] the pooled deviation of columns 0 .. 2,
 // out[1] that of column 3.  out[32] = 1: not usable.
 template <int Q, StatUse USE>
-__global__ void __launch_bounds__(ST) k_stats(long long n, const float* __restrict__ X, int vec,
+__global__ void __launch_bounds__(ST, 2) k_stats(long long n, const float* __restrict__ X, int vec,
                                               double* __restrict__ part, unsigned* done, double* __restrict__ out,
                                               float* __restrict__ norm) {
     constexpr int W = 4 * Q;
@@ -665,11 +683,11 @@ __global__ void __launch_bounds__(ST) k_stats(long long n, const float* __restri
     __syncthreads();
     const float s[4] = {shift[4 * q], shift[4 * q + 1], shift[4 * q + 2], shift[4 * q + 3]};
     double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};          // sums of columns 4q .. 4q+3, their squares
-    Pair a[8];
+    Triple a[8];
     const long long step = (long long)gridDim.x * (ST / Q);
     for (long long r = (long long)blockIdx.x * (ST / Q) + tid / Q; r < n; r += step * ST_FOLD) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) a[k] = {0.0f, 0.0f};
+        for (int k = 0; k < 8; ++k) a[k] = {0.0f, 0.0f, 0.0f};
 #pragma unroll 1
         for (int u0 = 0; u0 < ST_FOLD; u0 += 4) {
             if (r + step * u0 >= n) break;
@@ -684,16 +702,20 @@ __global__ void __launch_bounds__(ST) k_stats(long long n, const float* __restri
                 const float xs[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    Pair d = {xs[c], 0.0f};
-                    pair_add(d, -s[c], 0.0f);                         // x - s = d.h + d.l exactly
-                    pair_add(a[c], d.h, d.l);
-                    const float p = __fmul_rn(d.h, d.h);
-                    pair_add(a[4 + c], p, __fmaf_rn(2.0f * d.h, d.l, __fmaf_rn(d.h, d.h, -p)));
+                    float dl;
+                    const float dh = two_sum(xs[c], -s[c], dl);       // x - s = dh + dl exactly
+                    add(a[c], dh);
+                    add_low(a[c], dl);
+                    const float p = __fmul_rn(dh, dh), t = 2.0f * dh, q = __fmul_rn(t, dl);
+                    add(a[4 + c], p);
+                    add_low(a[4 + c], __fmaf_rn(dh, dh, -p));
+                    add_low(a[4 + c], q);
+                    a[4 + c].l = __fadd_rn(a[4 + c].l, __fmaf_rn(dl, dl, __fmaf_rn(t, dl, -q)));
                 }
             }
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] += (double)a[k].h + (double)a[k].l;
+        for (int k = 0; k < 8; ++k) v[k] += (double)a[k].h + ((double)a[k].m + (double)a[k].l);
     }
     // over the warp: each exchange halves the values a lane keeps, so lane l
     // ends with value 4 b4 + 2 b3 + b2 (its bits) of quad l % Q
@@ -745,7 +767,7 @@ __global__ void __launch_bounds__(ST) k_stats(long long n, const float* __restri
         const double off = s1 * s1 / cnt, dev = fmax(0.0, s2 - off);  // sum of squared deviations
         mean_s[tid] = (double)shift[tid] + s1 / cnt;
         dev_s[tid] = dev;
-        bad = !isfinite(s1) || !isfinite(s2) || off > 64.0 * dev;
+        bad = !isfinite(s1) || !isfinite(s2) || off > 4.0 * dev;
     }
     const bool any = __syncthreads_or(bad) != 0;
     if (USE == STAT_NORM) {

@@ -402,3 +402,21 @@ def test_statistics_wait_for_the_data(kind):
     torch.cuda.synchronize()
     if kind == "blocking":
         assert int(torch.cuda.cudart().cudaStreamDestroy(handle.value)) == 0
+
+
+@pytest.mark.parametrize("rows_per_thread", [1, 8, 32])
+def test_target_scales_hold_fp64_sums(rows_per_thread):
+    """Equal squares, whose rounding errors all have one sign, over a full fold
+    of every thread and less.  Sums in FP64 from a tree of 64 additions (fold,
+    warp, block, the blocks' partials) lose 64 x 2^-53 at most, the deviation
+    half of that; two more for the division and the root."""
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    n = rows_per_thread * 1024 * torch.cuda.get_device_properties(0).multi_processor_count
+    a = np.float32(float.fromhex("0x1.1f95f4p+0"))
+    T = torch.full((n, 4), float(a), device="cuda")
+    T[n // 2:] = -float(a)
+    _, sm, sp = MLP(seed=1).fit_target_scales(T)
+    for got, count in ((sm, 3 * n), (sp, n)):
+        want = np.longdouble(a) * np.sqrt(np.longdouble(count) / np.longdouble(count - 1))
+        assert abs(np.longdouble(got) / want - 1) <= 34 * 2.0 ** -53
