@@ -872,22 +872,30 @@ int fp64_blocks_per_sm(int nphi, int nsm) {
     return best;
 }
 
+// The kernel and the threads per block of a launch, the same for every entry
+// point: the caller's choice, the rule above for plain FP64, else the choice
+// made at upload.
+struct SolverLaunch {
+    const void* kernel;
+    int threads;
+};
+SolverLaunch solver_launch(const mm_ctx* ctx, int mode, int precision) {
+    const bool chosen = ctx->blocks_per_sm_req >= 2 && ctx->blocks_per_sm_req <= 4;     // by the caller
+    if (chosen || precision != 0 || (mode != mm::MODE_MINIMIZE && mode != mm::MODE_EVAL))
+        return {ctx->kernel, ctx->threads};
+    const int variant = fp64_blocks_per_sm(ctx->P.nphi, ctx->nsm);
+    return {mm::solver_kernel(variant), mm::solver_threads(variant)};
+}
+
 int launch_solver(mm_ctx* ctx, int mode, const mm::Params& prm) {
     ctx->P.prm = prm;
     ctx->P.mode = mode;
     CK_CUDA(cudaMemsetAsync(ctx->P.bar, 0, 64 * sizeof(unsigned), ctx->stream));
     CK_CUDA(cudaMemsetAsync(ctx->P.err, 0, sizeof(int), ctx->stream));
     void* args[] = {(void*)&ctx->P};
-    const void* kernel = ctx->kernel;
-    int threads = ctx->threads;
-    const bool chosen = ctx->blocks_per_sm_req >= 2 && ctx->blocks_per_sm_req <= 4;     // by the caller
-    if (!chosen && prm.precision == 0 && (mode == mm::MODE_MINIMIZE || mode == mm::MODE_EVAL)) {
-        const int variant = fp64_blocks_per_sm(ctx->P.nphi, ctx->nsm);
-        kernel = mm::solver_kernel(variant);
-        threads = mm::solver_threads(variant);
-    }
+    const SolverLaunch l = solver_launch(ctx, mode, prm.precision);
     CK_CUDA(cudaEventRecord(ctx->ev0, ctx->stream));
-    CK_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(ctx->blocks), dim3(threads), args, 0, ctx->stream));
+    CK_CUDA(cudaLaunchCooperativeKernel(l.kernel, dim3(ctx->blocks), dim3(l.threads), args, 0, ctx->stream));
     CK_CUDA(cudaEventRecord(ctx->ev1, ctx->stream));
     CK_CUDA(cudaMemcpyAsync(ctx->h_state, ctx->d_state, sizeof(mm::DevState), cudaMemcpyDeviceToHost,
                             ctx->stream));
@@ -1025,8 +1033,9 @@ int ctx_view(mm_ctx* ctx, CtxView* out) {
     out->node_of_phi = ctx->d_node_of_phi;
     out->ident = ctx->d_ident;
     out->has_mesh = ctx->has_mesh;
-    out->kernel = ctx->kernel;
-    out->threads = ctx->threads;
+    const SolverLaunch l = solver_launch(ctx, mm::MODE_EVAL, 0);
+    out->kernel = l.kernel;
+    out->threads = l.threads;
     out->d_state = ctx->d_state;
     out->nnz_mag = ctx->nnzm_true;
     out->nnz_phi = ctx->nnzp_true;

@@ -217,7 +217,7 @@ struct CtxView {
     const int* node_of_phi;      // device
     const unsigned char* ident;  // device
     bool has_mesh;
-    const void* kernel;          // the solver kernel the context launches
+    const void* kernel;          // the solver kernel of a plain FP64 evaluation
     int threads;                 // and its threads per block
     DevState* d_state;           // device
     long long nnz_mag, nnz_phi;  // true nonzeros of the two graphs

@@ -111,3 +111,37 @@ def test_noalloc_rejects_zero_and_nonfinite_vectors():
     F_ref, _ = mag.energy(wl.m0, Params(poisson_tol=1e-12))
     assert float(energy_dev[0].item()) == pytest.approx(F_ref, rel=1e-10)
     mag.close()
+
+
+@pytest.mark.parametrize("n_mag,variant", [(20, 2), (22, 3), (26, 4)])
+def test_fp64_entry_points_choose_the_same_launch(n_mag, variant):
+    """Plain FP64 runs with 512, 768 or 1024 threads per SM, chosen by the mesh
+    (these sizes: one each on 152 SMs), whichever entry point evaluates: the
+    no-allocation energy and gradient, the gradient and a minimisation are bit
+    by bit those of a context that asks for the same threads."""
+    import torch
+    from paper_1801_03690_gb300 import Magnet, Params
+    from paper_1801_03690_gb300 import _lib
+
+    lib = _lib.load()
+    wl = synth.small_cube(n_mag=n_mag, h=2.5e-9, seed=2)
+    prm = Params(poisson_tol=1e-10, max_iter=2)
+    pc = prm.to_c()
+    out = []
+    for bps in (0, variant):
+        mag = Magnet(device=0, blocks_per_sm=bps)
+        mag.upload_workload(wl)
+        mag.set_field(np.array([0.05, 0.0, 0.02]))
+        m_dev = torch.tensor(wl.m0, dtype=torch.float64, device="cuda")
+        grad_dev = torch.zeros_like(m_dev)
+        energy_dev = torch.zeros(5, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        rc = lib.mm_energy_gradient_noalloc(mag._h, C.c_void_p(m_dev.data_ptr()), C.byref(pc),
+                                            C.c_void_p(grad_dev.data_ptr()), 0, C.c_void_p(energy_dev.data_ptr()))
+        assert rc == 0, lib.mm_last_error(mag._h).decode()
+        g = mag.gradient(wl.m0, params=prm)
+        mag.set_magnetization(wl.m0)
+        mag.minimize(prm)
+        out.append((energy_dev.cpu().numpy(), grad_dev.cpu().numpy(), g, mag.get_magnetization()))
+        mag.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
