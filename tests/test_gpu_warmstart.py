@@ -420,3 +420,59 @@ def test_target_scales_hold_fp64_sums(rows_per_thread):
     for got, count in ((sm, 3 * n), (sp, n)):
         want = np.longdouble(a) * np.sqrt(np.longdouble(count) / np.longdouble(count - 1))
         assert abs(np.longdouble(got) / want - 1) <= 34 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 20011])
+def test_forward_on_odd_addresses(n):
+    """Inputs and outputs off a 16-byte boundary take scalar loads and stores;
+    the outputs are those of aligned arrays, bit by bit."""
+    import ctypes as C
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    net = MLP(seed=4)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn((n, 16), generator=g, device="cuda")
+    Y = net.forward(X)
+    xb, yb = torch.zeros(16 * n + 1, device="cuda"), torch.full((4 * n + 2,), 7.0, device="cuda")
+    xb[1:] = X.reshape(-1)
+    torch.cuda.synchronize()
+    for x, y in ((xb[1:], yb[1:-1]), (X, yb[1:-1]), (xb[1:], torch.empty(4 * n, device="cuda"))):
+        rc = net._lib.mm_mlp_forward(net._h, C.c_void_p(x.data_ptr()), n, C.c_void_p(y.data_ptr()))
+        assert rc == 0 and torch.equal(y.view(n, 4), Y)
+    assert yb[0] == 7.0 and yb[-1] == 7.0
+
+
+@pytest.mark.parametrize("path", [0, 1])
+@pytest.mark.parametrize("tiles", [0, 1, "sms"])
+def test_adam_steps_match_fp64(path, tiles):
+    """Training steps against Adam in FP64 from the gradient that each step has
+    (the same pass, without the update), at 1 row, one row more than a tile and
+    one more than a tile per SM; and the BF16 copies are those of the weights.
+    Per step a weight rounds once (2^-24 of itself, counted twice), and its
+    change, at most 1.1 lr in these four steps, has the rounding errors of the
+    moments, quotients and root (about ten of 2^-24) and that of 1 - beta2^k,
+    where the difference of two numbers near one keeps 7e-6: together below
+    2e-5 of 2 lr."""
+    import torch
+    from paper_1801_03690_gb300 import MLP
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 1 + 128 * (sms if tiles == "sms" else tiles)
+    net = MLP(seed=6)
+    net.set_tensor_path(path)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    lr, b1, b2 = np.float32(2e-3), float(np.float32(0.9)), float(np.float32(0.999))
+    p = net.get_params().astype(np.float64)
+    m, v = np.zeros_like(p), np.zeros_like(p)
+    for k in range(1, 5):
+        X, T = torch.randn((n, 16), generator=g, device="cuda"), torch.randn((n, 4), generator=g, device="cuda")
+        gr, loss = net.gradient(X, T)
+        assert net.train_step(X, T, float(lr), want_loss=True) == loss
+        gr = gr.astype(np.float64)
+        m, v = b1 * m + (1 - b1) * gr, b2 * v + (1 - b2) * gr * gr
+        p = p - float(lr) * (m / (1 - b1 ** k)) / (np.sqrt(v / (1 - b2 ** k)) + 1e-8)
+        got = net.get_params()
+        assert np.all(np.abs(got - p) <= k * (2.0 ** -23 * np.abs(p) + 2e-5 * 2 * float(lr)))
+    twin = MLP(seed=1)
+    twin.set_tensor_path(path)
+    twin.set_params(got)
+    assert torch.equal(net.forward(X), twin.forward(X))
