@@ -69,9 +69,11 @@ typedef struct {
 
 typedef struct {
     int device;           /* CUDA device ordinal                                 */
-    int blocks_per_sm;    /* solver kernel built for 2, 3 or 4 blocks/SM; 0 =    */
-                          /* chosen at mm_upload_mesh: 4 above 2 M potential    */
-                          /* unknowns, else 2                                   */
+    int blocks_per_sm;    /* threads per SM of the solver kernel in units of    */
+                          /* 256: 2, 3 or 4 (one block per SM); 0 = chosen: in  */
+                          /* plain FP64 evaluations and minimisations by the    */
+                          /* rounds of rows a launch takes, else 4 above 2 M    */
+                          /* potential unknowns and 2 below                     */
     void* stream;         /* cudaStream_t to run on; NULL = a private stream     */
 } mm_options;
 
@@ -416,7 +418,7 @@ int64_t mm_mlp_param_count(void);
 int mm_mlp_create(mm_mlp** mlp, int device, uint64_t seed);
 void mm_mlp_destroy(mm_mlp* mlp);
 int mm_mlp_set_params(mm_mlp* mlp, const float* params, int64_t count);
-/* Tensor-core path of the forward pass and of the weight gradients: 0
+/* Tensor-core path of the forward pass and of the training pass: 0
  * (default) = tcgen05 MMAs with FP32 accumulators in tensor memory (M = 128
  * per MMA), 1 = the warp-level mma.sync path, kept as a measured
  * comparison.  Both round at the same points (BF16 inputs, weights and

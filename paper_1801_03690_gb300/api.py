@@ -489,7 +489,7 @@ class MLP:
             raise MMError(rc, "mm_mlp_set_input_norm")
 
     def set_tensor_path(self, path):
-        """0: tcgen05 forward pass (default); 1: mma.sync (comparison)."""
+        """0: tcgen05 forward and training passes (default); 1: mma.sync (comparison)."""
         rc = self._lib.mm_mlp_set_tensor_path(self._h, int(path))
         if rc:
             raise MMError(rc, "mm_mlp_set_tensor_path")

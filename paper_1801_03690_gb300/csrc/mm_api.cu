@@ -838,12 +838,13 @@ int select_kernel(mm_ctx* ctx, int variant) {
     return MM_OK;
 }
 
-// Blocks per SM when the caller left the choice to the library: the phases
-// of a potential step are latency-bound, and on GB300 more resident warps
-// pay once the mesh is large -- 4 blocks per SM (64 registers) ran the
-// 8.7 M-unknown polycrystal 1.26x (multigrid precision form) and 1.30x
-// (plain FP64) faster than 2 -- while on the 0.86 M-unknown cube 2 blocks
-// per SM (128 registers, fewest spills) were fastest.
+// Threads per SM in units of 256 when the caller left the choice to the
+// library: the phases of a potential step are latency-bound, and on GB300 more
+// resident warps pay once the mesh is large, while on smaller ones the 128
+// registers at 2 x 256 threads (fewest spills) do.  Field steps in the
+// multigrid precision form at 2 / 3 / 4, ms: 493,039 unknowns (jittered cube)
+// 21.9 / 22.9 / 23.2, 857,375 30.6 / 30.5 / 31.2; graded polycrystals of
+// 1,771,561 56.1 / 54.8 / 56.8 and of 3,176,523 112.9 / 101.7 / 97.5.
 constexpr int kAutoLargePhi = 2000000;
 int auto_blocks_per_sm(int nphi) { return nphi > kAutoLargePhi ? 4 : 2; }
 
@@ -1102,9 +1103,10 @@ int mm_create(mm_ctx** out, const mm_options* opt) {
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
     if (!coop) return bail(MM_ERR_CUDA);
     cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, ctx->device);
-    // blocks_per_sm selects the kernel instantiation (register budget) and
-    // the grid: 2, 3 or 4 blocks per SM; 0 = chosen by mm_upload_mesh from
-    // the mesh size (select_kernel), 2 until then.
+    // blocks_per_sm selects the kernel instantiation: 2, 3 or 4 x 256 threads
+    // per SM with the registers that leaves, as one block; 0 = chosen by
+    // mm_upload_mesh from the mesh size (select_kernel), 2 until then, and per
+    // launch in plain FP64 (solver_launch).
     const int variant = (ctx->blocks_per_sm_req >= 2 && ctx->blocks_per_sm_req <= 4) ? ctx->blocks_per_sm_req : 2;
     if (select_kernel(ctx, variant) != MM_OK) return bail(MM_ERR_CUDA);
     if (opt && opt->stream) {

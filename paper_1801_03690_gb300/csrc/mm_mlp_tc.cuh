@@ -216,7 +216,7 @@ __device__ __forceinline__ void hidden_epilogue(unsigned char* hb, unsigned tlan
 // group waits for its product or runs its epilogue, the others' products keep
 // the tensor core at work.  Two CTAs of 128 threads, each with weights of its
 // own, element-wise staging and two-byte stores took 61 us a call at 20,011
-// rows and 615 us at 3,375,000; this form takes 45 and 356 (the tensor rate
+// rows and 615 us at 3,375,000; this form takes 41 and 350 (the tensor rate
 // would allow 123).
 __global__ void __launch_bounds__(GROUPS * TM, 1) k_mlp_forward_tc(long long n, const float* __restrict__ X, int vec,
                                                                    const __nv_bfloat16* __restrict__ wb,
@@ -369,8 +369,9 @@ __global__ void __launch_bounds__(GROUPS * TM, 1) k_mlp_forward_tc(long long n, 
 // separate kernels (forward, backward, and per layer a weight-gradient, a
 // reduction and a bias kernel, activations and dZ in HBM, two-byte strided
 // loads, the loss by one block) a training step took 222 / 333 / 957 us at
-// 64 / 16,384 / 65,536 rows; it takes 65 / 70 / 103 us now, with the
-// caller's reads of the loss and the parameters.
+// 64 / 16,384 / 65,536 rows; it takes 80 / 82 / 116 us now, with the
+// caller's reads of the loss and the parameters (31 us at 16,384 rows in a
+// loop that reads neither).
 constexpr int TT = 256;              // threads: two per row, each with half the columns
 constexpr int TRAIN_COLS = 512;      // TMEM columns allocated
 constexpr int C_G3 = 128, C_G2 = 256, C_G1 = 384, C_G4 = 400, C_B = 416;

@@ -145,10 +145,9 @@ __device__ __forceinline__ double fold_tree(double (&a)[N], bool sum) {
 }
 
 // Over the lanes of a warp; the result is lane 0's.
-template <int LANES = 32>
 __device__ __forceinline__ double warp_fold(double v, bool sum) {
 #pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) {
+    for (int o = 16; o > 0; o >>= 1) {
         const double u = __shfl_down_sync(0xffffffffu, v, o);
         v = sum ? v + u : fmax(v, u);
     }
