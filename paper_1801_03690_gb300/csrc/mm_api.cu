@@ -875,16 +875,20 @@ int fp64_blocks_per_sm(int nphi, int nsm) {
 
 // The kernel and the threads per block of a launch, the same for every entry
 // point: the caller's choice, the rule above for plain FP64, else the choice
-// made at upload.
+// made at upload.  Plain FP64 at 1024 threads takes the form for many rows above
+// kAutoLargePhi: field steps in the form for fewer rows / in this one, ms: graded
+// polycrystals of 2,146,689 unknowns 117.2 / 115.4, of 3,176,523 202.0 / 197.7, of
+// 5,000,211 365.3 / 346.4, a jittered cube of 2,048,383 131.9 / 122.7, a lattice
+// cube of as many 75.8 / 74.2, but one of 857,375 28.4 / 29.6.
 struct SolverLaunch {
     const void* kernel;
     int threads;
 };
 SolverLaunch solver_launch(const mm_ctx* ctx, int mode, int precision) {
     const bool chosen = ctx->blocks_per_sm_req >= 2 && ctx->blocks_per_sm_req <= 4;     // by the caller
-    if (chosen || precision != 0 || (mode != mm::MODE_MINIMIZE && mode != mm::MODE_EVAL))
-        return {ctx->kernel, ctx->threads};
-    const int variant = fp64_blocks_per_sm(ctx->P.nphi, ctx->nsm);
+    if (precision != 0 || (mode != mm::MODE_MINIMIZE && mode != mm::MODE_EVAL)) return {ctx->kernel, ctx->threads};
+    const int variant = chosen ? ctx->blocks_per_sm_req : fp64_blocks_per_sm(ctx->P.nphi, ctx->nsm);
+    if (variant == 4 && ctx->P.nphi > kAutoLargePhi) return {mm::solver_kernel_large(), mm::solver_threads(4)};
     return {mm::solver_kernel(variant), mm::solver_threads(variant)};
 }
 
@@ -1001,6 +1005,7 @@ namespace mm {
 const void* solver_kernel_2();
 const void* solver_kernel_3();
 const void* solver_kernel_4();
+const void* solver_kernel_4_large();
 const void* solver_batch_kernel_2();
 const void* solver_batch_kernel_3();
 const void* solver_batch_kernel_4();
@@ -1012,6 +1017,8 @@ const void* solver_kernel(int min_blocks) {
         default: return solver_kernel_3();
     }
 }
+
+const void* solver_kernel_large() { return solver_kernel_4_large(); }
 
 int solver_threads(int min_blocks) { return 256 * (min_blocks == 2 || min_blocks == 4 ? min_blocks : 3); }
 
@@ -1509,9 +1516,9 @@ int mm_upload_mesh(mm_ctx* ctx, int64_t n_nodes, const double* xyz, int64_t n_te
     if ((rc = build_hierarchy(ctx, P, std::move(Kfull)))) return rc;
     if (ctx->blocks_per_sm_req < 2 || ctx->blocks_per_sm_req > 4) {
         if (select_kernel(ctx, auto_blocks_per_sm(nphi)) != MM_OK) return fail(ctx, MM_ERR_CUDA, "no solver grid");
-        cudaFuncAttributes fa;           // loads the FP64 form's kernel here rather than in its first launch
-        CK_CUDA(cudaFuncGetAttributes(&fa, mm::solver_kernel(fp64_blocks_per_sm(nphi, ctx->nsm))));
     }
+    cudaFuncAttributes fa;               // loads the FP64 form's kernel here rather than in its first launch
+    CK_CUDA(cudaFuncGetAttributes(&fa, solver_launch(ctx, mm::MODE_EVAL, 0).kernel));
     if ((rc = dalloc(ctx, &P.partials, 2 * (size_t)MM_MAXRED * ctx->blocks))) return rc;
     if ((rc = dalloc(ctx, &P.bar, 64))) return rc;
     if ((rc = dalloc(ctx, &P.err, 1))) return rc;

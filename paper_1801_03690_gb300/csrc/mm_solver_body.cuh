@@ -17,6 +17,24 @@
 
 #include "mm_internal.cuh"
 
+// MM_LARGE 1: the form for plain FP64 on meshes of many rows (mm_kern_s4_large.cu),
+// where a potential step waits for memory rather than for the FP64 pipe.  There
+// the branches that skip the multiply-adds of padding, and the registers that
+// the minimiser's own state takes once it is inlined around the phases, keep
+// loads from being issued early: 8.7 M unknowns took 368 us a CG step in the
+// other form and 332 us in this one (without the branches or with the minimiser
+// a function of its own alone: 366 and 367), 3.2 M 146 and 135.  Below, the pipe
+// and the fixed costs of a phase count: the other form is faster on 250,047
+// unknowns (field step 26.1 against 27.9 ms) and on 29,791 (9.4 against 10.0).
+#ifndef MM_LARGE
+#define MM_LARGE 0
+#endif
+#if MM_LARGE
+#define MM_OUTLINE __noinline__
+#else
+#define MM_OUTLINE
+#endif
+
 namespace mm {
 
 namespace {
@@ -399,7 +417,7 @@ __device__ __forceinline__ T sell_dot_row(const Row& A, const int* __restrict__ 
 #pragma unroll
         for (int u = 0; u < CH; ++u) {
             const T g = (T)x[c[u]];
-            if (sizeof(T) == 4 || k0 + u < A.width) s += (T)v[u] * g;
+            if (MM_LARGE || sizeof(T) == 4 || k0 + u < A.width) s += (T)v[u] * g;
         }
     }
     return s;
@@ -424,6 +442,12 @@ __device__ __forceinline__ T sell_dot(const long long* __restrict__ sptr, const 
 // 250,047 rows of 15 entries).
 template <typename XT, class Pre, class F>
 __device__ __forceinline__ void phi_products(const Problem& P, const Team& t, const XT* x, Pre pre, F f) {
+#if MM_LARGE
+    for (int p = t.rank * MM_BLOCK + (int)threadIdx.x; p < P.nphi; p += t.nb * MM_BLOCK) {
+        const double s = sell_dot_row<8, double>(sell_row(P.p_sptr, p), P.p_col, P.Kp, x, p);
+        f(p, s, pre(p));
+    }
+#else
     const Share h = t.sm->phi;
     const int lane = threadIdx.x & 31;
     auto item = [&](int k) { return k <= h.full ? team_item(t, h, k) : -1; };
@@ -441,6 +465,7 @@ __device__ __forceinline__ void phi_products(const Problem& P, const Team& t, co
         i = ni;
         A = N;
     }
+#endif
 }
 struct NoOperands {};
 struct Operands {
@@ -1774,7 +1799,7 @@ __device__ __forceinline__ bool cubic_step(double f0, double g0, double a, doubl
 }
 
 // Algorithm 4 at the current field from slot C.cur.
-__device__ int minimize(Ctx& C, int& cur) {
+__device__ MM_OUTLINE int minimize(Ctx& C, int& cur) {
     const Problem& P = *C.P;
     const Params& prm = P.prm;
     int c = cur;
@@ -1963,7 +1988,7 @@ __device__ __forceinline__ void solver_body(const Problem& P, int nb, int rank) 
 // barrier of 152 blocks costs 1.25 us where one of 304 costs 1.42 us and one
 // of 608 2.28 us, and a reduction folds 152 partials.  Batches keep blocks of
 // 256 threads, so that small members can have a fraction of an SM.
-template <int MINB>
+template <int MINB, int LARGE = MM_LARGE>
 __global__ void __launch_bounds__(MM_BLOCK, MINB * 256 / MM_BLOCK) k_solver(const __grid_constant__ Problem P) {
     solver_body(P, (int)gridDim.x, (int)blockIdx.x);
 }

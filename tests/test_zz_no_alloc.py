@@ -145,3 +145,26 @@ def test_fp64_entry_points_choose_the_same_launch(n_mag, variant):
         out.append((energy_dev.cpu().numpy(), grad_dev.cpu().numpy(), g, mag.get_magnetization()))
         mag.close()
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("n_mag,large", [(62, False), (63, True)])
+def test_fp64_form_for_many_rows(n_mag, large):
+    """Above 2 M potential unknowns plain FP64 runs the form for many rows, with
+    the threads it chooses (4 x 256 here) and with those asked for: the same bits.
+    The gradient is that of 3 x 256 threads in the other form, both with the
+    potential solved to 1e-12; a residual enters it amplified by the square root of
+    the condition number, below 300 for the Jacobi-scaled operator on these
+    lattices: bound 1e-9 of the largest."""
+    from paper_1801_03690_gb300 import Magnet, Params
+
+    wl = synth.small_cube(n_mag=n_mag, h=2.5e-9, seed=2)
+    grads = []
+    for bps in (0, 4, 3):
+        mag = Magnet(device=0, blocks_per_sm=bps)
+        mag.upload_workload(wl)
+        assert (mag.sizes()["n_phi"] > 2000000) == large
+        mag.set_field(np.array([0.05, 0.0, 0.02]))
+        grads.append(mag.gradient(wl.m0, params=Params(poisson_tol=1e-12)))
+        mag.close()
+    assert np.array_equal(grads[0], grads[1])
+    assert np.abs(grads[0] - grads[2]).max() <= 1e-9 * np.abs(grads[2]).max()
