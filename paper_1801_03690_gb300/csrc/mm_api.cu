@@ -875,11 +875,15 @@ int fp64_blocks_per_sm(int nphi, int nsm) {
 
 // The kernel and the threads per block of a launch, the same for every entry
 // point: the caller's choice, the rule above for plain FP64, else the choice
-// made at upload.  Plain FP64 at 1024 threads takes the form for many rows above
-// kAutoLargePhi: field steps in the form for fewer rows / in this one, ms: graded
+// made at upload.  Plain FP64 takes the form for many rows above kManyRows.  Field
+// steps in the form for fewer rows / in this one, ms, at 4 x 256 threads: graded
 // polycrystals of 2,146,689 unknowns 117.2 / 115.4, of 3,176,523 202.0 / 197.7, of
 // 5,000,211 365.3 / 346.4, a jittered cube of 2,048,383 131.9 / 122.7, a lattice
-// cube of as many 75.8 / 74.2, but one of 857,375 28.4 / 29.6.
+// cube of as many 75.8 / 74.2, but one of 857,375 28.4 / 29.4.  At 2 and 3 x 256
+// the line lies lower: 493,039 unknowns (jittered) 32.6 / 25.5 and 28.2 / 25.3,
+// 857,375 59.0 / 45.1 and 48.6 / 42.6, 456,533 (graded) 21.7 / 20.0 and 19.6 / 19.6,
+// but on 166,375 (lattice) 8.4 / 8.0 and 7.8 / 8.1.
+constexpr int kManyRows[3] = {400000, 400000, 2000000};     // at 2, 3 and 4 x 256 threads
 struct SolverLaunch {
     const void* kernel;
     int threads;
@@ -888,8 +892,7 @@ SolverLaunch solver_launch(const mm_ctx* ctx, int mode, int precision) {
     const bool chosen = ctx->blocks_per_sm_req >= 2 && ctx->blocks_per_sm_req <= 4;     // by the caller
     if (precision != 0 || (mode != mm::MODE_MINIMIZE && mode != mm::MODE_EVAL)) return {ctx->kernel, ctx->threads};
     const int variant = chosen ? ctx->blocks_per_sm_req : fp64_blocks_per_sm(ctx->P.nphi, ctx->nsm);
-    if (variant == 4 && ctx->P.nphi > kAutoLargePhi) return {mm::solver_kernel_large(), mm::solver_threads(4)};
-    return {mm::solver_kernel(variant), mm::solver_threads(variant)};
+    return {mm::solver_kernel(variant, ctx->P.nphi > kManyRows[variant - 2]), mm::solver_threads(variant)};
 }
 
 int launch_solver(mm_ctx* ctx, int mode, const mm::Params& prm) {
@@ -1005,20 +1008,20 @@ namespace mm {
 const void* solver_kernel_2();
 const void* solver_kernel_3();
 const void* solver_kernel_4();
+const void* solver_kernel_2_large();
+const void* solver_kernel_3_large();
 const void* solver_kernel_4_large();
 const void* solver_batch_kernel_2();
 const void* solver_batch_kernel_3();
 const void* solver_batch_kernel_4();
 
-const void* solver_kernel(int min_blocks) {
+const void* solver_kernel(int min_blocks, bool many_rows) {
     switch (min_blocks) {
-        case 2: return solver_kernel_2();
-        case 4: return solver_kernel_4();
-        default: return solver_kernel_3();
+        case 2: return many_rows ? solver_kernel_2_large() : solver_kernel_2();
+        case 4: return many_rows ? solver_kernel_4_large() : solver_kernel_4();
+        default: return many_rows ? solver_kernel_3_large() : solver_kernel_3();
     }
 }
-
-const void* solver_kernel_large() { return solver_kernel_4_large(); }
 
 int solver_threads(int min_blocks) { return 256 * (min_blocks == 2 || min_blocks == 4 ? min_blocks : 3); }
 

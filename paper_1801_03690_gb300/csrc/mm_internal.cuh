@@ -230,9 +230,8 @@ namespace mm {
 // Device function pointer of the solver kernel built for at least
 // min_blocks x 256 resident threads per SM (2, 3 or 4; others -> 3), and the
 // threads per block it is launched with (min_blocks x 256: one block per SM).
-const void* solver_kernel(int min_blocks);
-// The one of 4 x 256 threads in the form for plain FP64 on many rows.
-const void* solver_kernel_large();
+// many_rows: in the form for plain FP64 on many rows.
+const void* solver_kernel(int min_blocks, bool many_rows = false);
 int solver_threads(int min_blocks);
 // The batched solver kernel (teams of blocks, one problem per team);
 // min_blocks 3 or 4 (others -> 3).

@@ -17,13 +17,13 @@
 
 #include "mm_internal.cuh"
 
-// MM_LARGE 1: the form for plain FP64 on meshes of many rows (mm_kern_s4_large.cu),
+// MM_LARGE 1: the form for plain FP64 on meshes of many rows (mm_kern_s*_large.cu),
 // where a potential step waits for memory rather than for the FP64 pipe.  There
 // the branches that skip the multiply-adds of padding, and the registers that
 // the minimiser's own state takes once it is inlined around the phases, keep
 // loads from being issued early: 8.7 M unknowns took 368 us a CG step in the
 // other form and 332 us in this one (without the branches or with the minimiser
-// a function of its own alone: 366 and 367), 3.2 M 146 and 135.  Below, the pipe
+// a function of its own alone: 366 and 367), 3.2 M 146 and 135 (1024 threads).  Below, the pipe
 // and the fixed costs of a phase count: the other form is faster on 250,047
 // unknowns (field step 26.1 against 27.9 ms) and on 29,791 (9.4 against 10.0).
 #ifndef MM_LARGE

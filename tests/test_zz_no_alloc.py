@@ -168,3 +168,23 @@ def test_fp64_form_for_many_rows(n_mag, large):
         mag.close()
     assert np.array_equal(grads[0], grads[1])
     assert np.abs(grads[0] - grads[2]).max() <= 1e-9 * np.abs(grads[2]).max()
+
+
+@pytest.mark.parametrize("n_mag,many", [(36, False), (38, True)])
+def test_fp64_forms_agree_at_fewer_threads(n_mag, many):
+    """At 2 and 3 x 256 threads the form for many rows begins at 400,000 potential
+    unknowns: the gradient on either side of that against 4 x 256 threads, which
+    still run the other form there.  Bound as in the test above."""
+    from paper_1801_03690_gb300 import Magnet, Params
+
+    wl = synth.small_cube(n_mag=n_mag, h=2.5e-9, seed=2)
+    grads = []
+    for bps in (4, 2, 3):
+        mag = Magnet(device=0, blocks_per_sm=bps)
+        mag.upload_workload(wl)
+        assert (mag.sizes()["n_phi"] > 400000) == many
+        mag.set_field(np.array([0.05, 0.0, 0.02]))
+        grads.append(mag.gradient(wl.m0, params=Params(poisson_tol=1e-12)))
+        mag.close()
+    for g in grads[1:]:
+        assert np.abs(g - grads[0]).max() <= 1e-9 * np.abs(grads[0]).max()
