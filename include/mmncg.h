@@ -450,16 +450,16 @@ int mm_mlp_train_step(mm_mlp* mlp, const float* X_dev, const float* T_dev, int64
 /* Set the input standardisation from data: per feature, the mean and the
  * unbiased standard deviation of X_dev [n][16] (device; sums of FP64
  * precision or better, blocks in a fixed order); a feature whose deviation is below 1e-6 (|mean| + 1)
- * is only centred.  Waits for the work that the default stream, and the
- * streams that block on it, have been given.  n >= 2.  mm_mlp_get_input_norm reads back the mean and
+ * is only centred.  Runs behind the work that the default stream, and the
+ * streams that block on it, have been given, and waits for it.  n >= 2.  mm_mlp_get_input_norm reads back the mean and
  * 1/std in use. */
 int mm_mlp_fit_input_norm(mm_mlp* mlp, const float* X_dev, int64_t n);
 int mm_mlp_get_input_norm(mm_mlp* mlp, float mean[16], float inv_stdev[16]);
 /* Target scales for training: *scale_m = the unbiased standard deviation of
  * the m-columns T[:, 0:3] taken together, *scale_phi that of T[:, 3] (each
  * at least 1e-12), and Tn_dev [n][4] = T_dev with those columns divided by
- * them (device arrays; Tn_dev may be T_dev).  Waits as
- * mm_mlp_fit_input_norm does.  n >= 2. */
+ * them (device arrays; Tn_dev may be T_dev).  Runs and
+ * waits as mm_mlp_fit_input_norm does.  n >= 2. */
 int mm_mlp_fit_target_scales(mm_mlp* mlp, const float* T_dev, int64_t n, float* Tn_dev, double* scale_m,
                              double* scale_phi);
 /* Training targets of one field step from the features of the converged

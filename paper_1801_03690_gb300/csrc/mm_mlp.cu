@@ -624,9 +624,9 @@ __global__ void k_ws_targets(long long n, const float* __restrict__ X0, const fl
 // 2^-53 of the sum of magnitudes, where 32 FP64 additions may lose 32 times
 // that.  It takes 60 FP32 operations an element.  (Two words take 24 but hold
 // about 43 bits: equal squares in 4,980,736 rows gave a deviation off by 9e-14.)
-// Standardising and scaling a training set of 1,200,003 rows takes 196 us with
+// Standardising and scaling a training set of 1,200,003 rows takes 184 us with
 // two blocks resident per SM (64 registers, 112 B spilled outside the row loop;
-// 209 with one), 802 with the FP64 passes and their work space per call.  The
+// 13 us more with one), 797 with the FP64 passes and their work space per call.  The
 // target scales come out within 2.3 x 2^-53 of 64-bit ones at 1,000 to 3,000,000
 // rows (FP64 passes: within 7.9 x 2^-53).
 // A result that is not finite (the FP32 squares overflow above 1e19) goes to
@@ -1257,12 +1257,17 @@ int mm_mlp_train_step(mm_mlp* M, const float* X_dev, const float* T_dev, int64_t
 
 namespace {
 
+// The statistics run on the default stream: behind what it and the streams that
+// block on it have been given, and behind the training steps so far, which it
+// waits for (before_caller).
+const cudaStream_t kStatStream = cudaStreamLegacy;
+
 // k_stats over an [n][4 Q] array.
 template <int Q, StatUse USE>
 int launch_stats(mm_mlp* M, const float* X, long long n) {
     const int grid = (int)std::min((n * Q + ST - 1) / ST, (long long)stat_blocks(M));
     const int vec = reinterpret_cast<uintptr_t>(X) % 16 == 0;
-    k_stats<Q, USE><<<grid, ST, 0, M->stream>>>(n, X, vec, M->stats + ST_OUT + 1,
+    k_stats<Q, USE><<<grid, ST, 0, kStatStream>>>(n, X, vec, M->stats + ST_OUT + 1,
                                                 reinterpret_cast<unsigned*>(M->stats + ST_OUT), M->stats, M->norm);
     MK(cudaGetLastError());
     return MM_OK;
@@ -1322,12 +1327,11 @@ extern "C" {
 int mm_mlp_fit_input_norm(mm_mlp* M, const float* X_dev, int64_t n) {
     if (!M || !X_dev || n < 2) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    int rc = after_caller(M);
+    int rc = launch_stats<NIN / 4, STAT_NORM>(M, X_dev, n);
     if (rc) return rc;
-    if ((rc = launch_stats<NIN / 4, STAT_NORM>(M, X_dev, n))) return rc;
     double flag;
-    MK(cudaMemcpyAsync(&flag, M->stats + 32, sizeof(flag), cudaMemcpyDeviceToHost, M->stream));
-    MK(cudaStreamSynchronize(M->stream));
+    MK(cudaMemcpyAsync(&flag, M->stats + 32, sizeof(flag), cudaMemcpyDeviceToHost, kStatStream));
+    MK(cudaStreamSynchronize(kStatStream));
     if (flag == 0.0) return MM_OK;
     double mean[NIN], sd[NIN];
     if ((rc = col_mean_std(M, X_dev, n, NIN, 0, NIN, 0, mean, sd))) return rc;
@@ -1359,15 +1363,14 @@ int mm_mlp_fit_target_scales(mm_mlp* M, const float* T_dev, int64_t n, float* Tn
                              double* scale_phi) {
     if (!M || !T_dev || !Tn_dev || !scale_m || !scale_phi || n < 2) return MM_ERR_ARG;
     MK(cudaSetDevice(M->device));
-    int rc = after_caller(M);
+    int rc = launch_stats<1, STAT_TARGETS>(M, T_dev, n);
     if (rc) return rc;
-    if ((rc = launch_stats<1, STAT_TARGETS>(M, T_dev, n))) return rc;
     const int vec = (reinterpret_cast<uintptr_t>(T_dev) | reinterpret_cast<uintptr_t>(Tn_dev)) % 16 == 0;
-    k_scale_by<<<(unsigned)((n + 255) / 256), 256, 0, M->stream>>>(n, T_dev, vec, M->stats, Tn_dev);
+    k_scale_by<<<(unsigned)((n + 255) / 256), 256, 0, kStatStream>>>(n, T_dev, vec, M->stats, Tn_dev);
     MK(cudaGetLastError());
     double h[33];
-    MK(cudaMemcpyAsync(h, M->stats, sizeof(h), cudaMemcpyDeviceToHost, M->stream));
-    MK(cudaStreamSynchronize(M->stream));
+    MK(cudaMemcpyAsync(h, M->stats, sizeof(h), cudaMemcpyDeviceToHost, kStatStream));
+    MK(cudaStreamSynchronize(kStatStream));
     if (h[32] == 0.0) {
         *scale_m = h[0];
         *scale_phi = h[1];

@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(GROUPS * TM, 1) k_mlp_forward_tc(long long n, 
 // separate kernels (forward, backward, and per layer a weight-gradient, a
 // reduction and a bias kernel, activations and dZ in HBM, two-byte strided
 // loads, the loss by one block) a training step took 222 / 333 / 957 us at
-// 64 / 16,384 / 65,536 rows; it takes 80 / 82 / 116 us now, with the
+// 64 / 16,384 / 65,536 rows; it takes 73 / 76 / 110 us now, with the
 // caller's reads of the loss and the parameters (31 us at 16,384 rows in a
 // loop that reads neither).
 constexpr int TT = 256;              // threads: two per row, each with half the columns
