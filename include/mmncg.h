@@ -449,10 +449,11 @@ int mm_mlp_train_step(mm_mlp* mlp, const float* X_dev, const float* T_dev, int64
                       float lr, float* loss_out);
 /* Set the input standardisation from data: per feature, the mean and the
  * unbiased standard deviation of X_dev [n][16] (device; sums of FP64
- * precision or better, blocks in a fixed order); a feature whose deviation is below 1e-6 (|mean| + 1)
- * is only centred.  Runs behind the work that the default stream, and the
- * streams that block on it, have been given, and waits for it.  n >= 2.  mm_mlp_get_input_norm reads back the mean and
- * 1/std in use. */
+ * precision or better, blocks in a fixed order); a feature whose deviation
+ * is below 1e-6 (|mean| + 1) is only centred.  Runs behind the work that the
+ * default stream, and the streams that block on it, have been given, and
+ * waits for it.  n >= 2.  mm_mlp_get_input_norm reads back the mean and 1/std
+ * in use. */
 int mm_mlp_fit_input_norm(mm_mlp* mlp, const float* X_dev, int64_t n);
 int mm_mlp_get_input_norm(mm_mlp* mlp, float mean[16], float inv_stdev[16]);
 /* Target scales for training: *scale_m = the unbiased standard deviation of
